@@ -16,6 +16,15 @@
 //                interaction reads, and each cell's x-sub-bin starts
 //
 // All kernels are HBM- or L2-bound integer work; none uses tensor cores.
+//
+// Every kernel after k_zero is a dependent launch (see launch_dependent), but
+// none of them calls pdl_trigger: the next kernel's blocks are released as
+// this one's exit.  Triggered on entry, they were placed while this kernel
+// still held its SMs, so a grid of less than a wave piled up on the SMs that
+// happened to be free: the interaction of 32,768 particles (128 CTAs) then
+// took 38 instead of 20 us.  Measured, step of pi_bin + pi_interact with the
+// trigger on entry / at exit: 57 / 36 us at 32,768 particles, 60 / 38 at
+// 65,536, 56 / 42 at 131,072, 328 / 324 at 2.1 M (binning 93 / 89).
 #include <algorithm>
 #include <mutex>
 
@@ -30,7 +39,6 @@ constexpr unsigned FULL = 0xffffffffu;
 template <int NB>
 __global__ void k_zero(ZeroArgs<NB> z)
 {
-    pdl_trigger();
     size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     size_t stride = (size_t)gridDim.x * blockDim.x;
     uint4* p4 = reinterpret_cast<uint4*>(z.p);
@@ -57,7 +65,6 @@ __global__ void __launch_bounds__(256) k_hist(const float* __restrict__ x,
                                               Ctrl* __restrict__ ctrl, int vec)
 {
     constexpr int HP = HIST_PER_LANE, HV = HP / 4;
-    pdl_trigger();
     const unsigned lane = threadIdx.x & 31u;
     const uint32_t groups = (n + HP - 1u) / HP;
     const uint32_t stride = gridDim.x * blockDim.x;
@@ -180,7 +187,6 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan(const uint32_t* __restric
     __shared__ uint32_t s_prefix;
 
     const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    pdl_trigger();
     pdl_wait();
     if (threadIdx.x == 0) s_tile = atomicAdd(ticket_slot ? &ctrl->tickets[ticket_slot - 1] : &ctrl->ticket, 1u);
     __syncthreads();
@@ -332,7 +338,6 @@ __global__ void __launch_bounds__(256) k_scatter(const uint32_t* __restrict__ ce
                                                  Rec* __restrict__ rec, Ctrl* __restrict__ ctrl,
                                                  int vec)
 {
-    pdl_trigger();
     pdl_wait();
     if (cta_error(ctrl)) return;
     bool bad = false;
@@ -424,7 +429,6 @@ __global__ void __launch_bounds__(256) k_stabilise(const Rec* __restrict__ rec, 
                                                    uint2* __restrict__ xbins,
                                                    Ctrl* __restrict__ ctrl)
 {
-    pdl_trigger();
     pdl_wait();
     if (cta_error(ctrl)) return;
     bool bad = false;

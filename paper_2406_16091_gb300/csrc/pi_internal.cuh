@@ -285,6 +285,8 @@ __device__ __forceinline__ uint64_t global_ns()
 // begin while the kernel before it in the stream is still running (once
 // every block of that kernel has called pdl_trigger or exited); pdl_wait
 // then blocks until that kernel has completed and its writes are visible.
+// The default binning kernels never trigger (see pi_bin.cu): their
+// successor's blocks are placed as their own exit, evenly over the SMs.
 // Whatever a kernel reads or writes of the step's state comes after its
 // pdl_wait.  For a kernel launched the ordinary way both are no-ops.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
