@@ -95,8 +95,9 @@ enum {
      * 768, 1280, 2432 staged particles; 3, 4 for the warp-specialised form
      * (one producer warp stages chunks of up to 2432 particles into 2
      * buffers for 4 or 8 consumer warps); 5 for the direct form (no
-     * staging: one thread per target pair reads its sources from global
-     * memory through L1; every kernel K and both precision modes); 6 for the
+     * staging: one thread per target pair -- per target for small systems
+     * and the costlier kernels -- reads its sources from global memory
+     * through L1; every kernel K and both precision modes); 6 for the
      * direct form with four targets per thread (fewer source reads per
      * evaluation, more evaluations: faster at high occupancy).  With a
      * kernel other than the Gaussian, shapes 0 - 4 all run shape 2's
@@ -124,7 +125,8 @@ enum {
      * of four-source trips included -- into a device counter that
      * pi_eval_count reads; 0 (default) counts nothing.  The copy exists for
      * the Gaussian kernel in PI_PREC_FP32 (the windows, and so the count,
-     * depend on the positions and r_c only); other kernels, the Kahan mode,
+     * depend on the positions and r_c only; shape 5 counts in its form with
+     * two targets per thread); other kernels, the Kahan mode,
      * the staged shapes, Alg. 1 and pi_autotune's timed trials count
      * nothing.  The count restarts at every pi_bin.  Results do not depend
      * on it. */

@@ -787,6 +787,33 @@ pi_status launch_plan(pi_ctx* ctx, pi::InteractArgs a, bool kahan, cudaStream_t 
     return PI_OK;
 }
 
+// Whether shape 5 takes one target per thread (k_interact_direct1) instead
+// of two.  Medians of the interaction in us, two targets / one (particles,
+// mean per cell):
+//   - few particles: one thread's chain of trips sets the time, and one
+//     target halves it, up to about 256 threads per SM of the plain and the
+//     compensated sums (Gaussian: 1,531 at 6 18.4 / 14.4, 10,000 at 8 22.5 /
+//     16.4, 32,768 at 8 20.5 / 18.4, 65,536 at 8 22.5 / 24.6) and 1024 of
+//     the costlier kernels (Lennard-Jones at 8: 30,000 34.8 / 24.6, 131,072
+//     45.1 / 38.9, 262,144 61.4 / 65.5);
+//   - the 168-FLOP kernel spends most on each evaluation, and one target
+//     has fewer of them: 465 / 375 and 975 / 922 (2 M at 2 and 8), dense
+//     clusters 2540 / 2132 (300,000 at 16);
+//   - the compensated exponent likewise below 16 per cell: 242 / 213, 473 /
+//     469 and 1436 / 1464 (2 M at 2, 8 and 32);
+//   - the compensated sums below 4 per cell: 211 / 203, 406 / 410 and 1221 /
+//     1251 (2 M at 2, 8 and 32), clustered 690 / 627 (1 M at 2) and 287 /
+//     317 (100,000 at 16).
+bool one_target_form(const pi_ctx* ctx, int kernel)
+{
+    const bool kahan = ctx->precision == PI_PREC_KAHAN;
+    const bool plain = !kahan && (kernel == pi::KERNEL_GAUSSIAN || kernel == pi::KERNEL_LOWFLOP);
+    if (ctx->n <= (int64_t)ctx->num_sms * (plain || kahan ? 256 : 1024)) return true;
+    if (kahan) return ctx->n < 4 * ctx->C;
+    if (kernel == pi::KERNEL_GAUSSIAN_FINE) return ctx->n < 16 * ctx->C;
+    return kernel == pi::KERNEL_HIGHFLOP;
+}
+
 // Occupancy regimes of the per-system autotuning: mean particles per cell
 // below 4, below 8, and from 8 on (the shapes' crossover is near 8).
 int occupancy_regime(const pi_ctx* ctx, int s)
@@ -874,6 +901,7 @@ pi_status pi_batch_interact(pi_ctx* ctx, const float* h, float* S, float* Vx, fl
     a.wait_limit_ns = ctx->wait_limit_ns;
     a.seq = ctx->tiled_seq;
     a.count_evals = ctx->count_evals;
+    a.one_target = one_target_form(ctx, a.kernel);
     int launched = 0;
     cudaError_t e;
     const bool kahan = ctx->precision == PI_PREC_KAHAN;

@@ -32,7 +32,9 @@
 //   k_interact_direct  (default) one thread per target pair, windows from
 //                      global memory, sources read through L1; one flattened
 //                      loop over all windows.  Every kernel K and both
-//                      precision modes.
+//                      precision modes.  k_interact_direct1 is its form with
+//                      one target per thread, k_interact_direct4 the one with
+//                      four.
 //   k_interact_tiled   work items are segments of an X-row of target cells,
 //                      handed out dynamically from one queue over all
 //                      systems and processed in chunks of consecutive cells;
@@ -730,6 +732,37 @@ __device__ __forceinline__ float2 gauss_fine2(float2 dx, float2 dy, float2 dz, f
     return __ffma2_rn(__fmul2_rn(k0, c), make_float2(LN2_F, LN2_F), k0);
 }
 
+// Two kernel values with packed FP32 arithmetic, each element rounded as
+// kernel_value's scalar steps round it, times the pair tests' 1/0 masks m.
+template <int KERNEL>
+__device__ __forceinline__ float2 packed_value(float2 dx, float2 dy, float2 dz, float2 r2, float2 m, float2 ks,
+                                               const KParams& kp)
+{
+    float2 K;
+    if constexpr (KERNEL == KERNEL_GAUSSIAN) {
+        const float2 t = __fmul2_rn(r2, ks);
+        K = __fmul2_rn(make_float2(ex2_approx(t.x), ex2_approx(t.y)), m);
+    } else if constexpr (KERNEL == KERNEL_GAUSSIAN_FINE) {
+        K = __fmul2_rn(gauss_fine2(dx, dy, dz, ks, make_float2(kp.tl, kp.tl)), m);
+    } else if constexpr (KERNEL == KERNEL_LOWFLOP) {
+        K = m;
+    } else {
+        // kernel_value's Lennard-Jones steps, element by element
+        const float2 rs2 = __ffma2_rn(make_float2(0.01f, 0.01f), ks, r2);
+        const float2 sr = __fmul2_rn(ks, make_float2(__frcp_rn(rs2.x), __frcp_rn(rs2.y)));
+        const float2 s3 = __fmul2_rn(__fmul2_rn(sr, sr), sr);
+        const float2 q = __ffma2_rn(s3, make_float2(-1.f, -1.f), __fmul2_rn(s3, s3));
+        float2 e = __fmul2_rn(make_float2(4.0f, 4.0f), q);
+        if constexpr (KERNEL == KERNEL_HIGHFLOP) {
+            const float2 one = make_float2(kp.one, kp.one), zero = make_float2(kp.zero, kp.zero);
+#pragma unroll
+            for (int i = 0; i < 75; ++i) e = __ffma2_rn(e, one, zero);
+        }
+        K = __fmul2_rn(e, m);
+    }
+    return K;
+}
+
 template <class Acc, int KERNEL>
 struct PairSumsT {
     static constexpr bool kahan = std::is_same<Acc, KahanAcc>::value;
@@ -761,28 +794,7 @@ struct PairSumsT {
         const float2 dz = __fadd2_rn(make_float2(p.z, p.z), make_float2(-ta.z, -tb.z));
         const float2 r2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
         const float2 m = make_float2(lt_ne_mask(r2.x, rc2, p.w, ta.w), lt_ne_mask(r2.y, rc2, p.w, tb.w));
-        float2 K;
-        if constexpr (KERNEL == KERNEL_GAUSSIAN) {
-            const float2 t = __fmul2_rn(r2, ks);
-            K = __fmul2_rn(make_float2(ex2_approx(t.x), ex2_approx(t.y)), m);
-        } else if constexpr (KERNEL == KERNEL_GAUSSIAN_FINE) {
-            K = __fmul2_rn(gauss_fine2(dx, dy, dz, ks, make_float2(kp.tl, kp.tl)), m);
-        } else if constexpr (KERNEL == KERNEL_LOWFLOP) {
-            K = m;
-        } else {
-            // kernel_value's Lennard-Jones steps, element by element
-            const float2 rs2 = __ffma2_rn(make_float2(0.01f, 0.01f), ks, r2);
-            const float2 sr = __fmul2_rn(ks, make_float2(__frcp_rn(rs2.x), __frcp_rn(rs2.y)));
-            const float2 s3 = __fmul2_rn(__fmul2_rn(sr, sr), sr);
-            const float2 q = __ffma2_rn(s3, make_float2(-1.f, -1.f), __fmul2_rn(s3, s3));
-            float2 e = __fmul2_rn(make_float2(4.0f, 4.0f), q);
-            if constexpr (KERNEL == KERNEL_HIGHFLOP) {
-                const float2 one = make_float2(kp.one, kp.one), zero = make_float2(kp.zero, kp.zero);
-#pragma unroll
-                for (int i = 0; i < 75; ++i) e = __ffma2_rn(e, one, zero);
-            }
-            K = __fmul2_rn(e, m);
-        }
+        const float2 K = packed_value<KERNEL>(dx, dy, dz, r2, m, ks, kp);
         if constexpr (!kahan) {
             s = __fadd2_rn(s, K);
             vx = __ffma2_rn(dx, K, vx);
@@ -1655,6 +1667,130 @@ __global__ void __launch_bounds__(DIRECT_THREADS, (direct_min_blocks<Acc, KERNEL
         direct_slot_pair<DIRECT_THREADS, false, Acc, KERNEL, COUNT>(a, win, threadIdx.x, k0, kend);
 }
 
+// ---- one target per thread ----
+//
+// Two candidate sources p and q of one target with packed arithmetic; the
+// sums take the two terms one after the other, rounded as the sequential
+// loop rounds them.
+template <int KERNEL, class Acc>
+__device__ __forceinline__ void cand_sources(const float4& p, const float4& q, const float4& t, float rc2, float2 ks,
+                                             const KParams& kp, Sums<Acc, KERNEL>& r, float& n)
+{
+    const float2 dx = __fadd2_rn(make_float2(p.x, q.x), make_float2(-t.x, -t.x));
+    const float2 dy = __fadd2_rn(make_float2(p.y, q.y), make_float2(-t.y, -t.y));
+    const float2 dz = __fadd2_rn(make_float2(p.z, q.z), make_float2(-t.z, -t.z));
+    const float2 r2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
+    const float2 m = make_float2(lt_ne_mask(r2.x, rc2, p.w, t.w), lt_ne_mask(r2.y, rc2, q.w, t.w));
+    const float2 K = packed_value<KERNEL>(dx, dy, dz, r2, m, ks, kp);
+    r.s.add(K.x, m.x != 0.f);
+    r.vx.addmul(dx.x, K.x, m.x != 0.f);
+    r.vy.addmul(dy.x, K.x, m.x != 0.f);
+    r.vz.addmul(dz.x, K.x, m.x != 0.f);
+    r.s.add(K.y, m.y != 0.f);
+    r.vx.addmul(dx.y, K.y, m.y != 0.f);
+    r.vy.addmul(dy.y, K.y, m.y != 0.f);
+    r.vz.addmul(dz.y, K.y, m.y != 0.f);
+    n += m.x;
+    n += m.y;
+}
+
+// The windows of direct_group for one target, four sources per trip.
+template <int WT, bool DENSE, class Acc, int KERNEL>
+__device__ __forceinline__ void direct_single(const InteractArgs& a, uint32_t (*win)[WT], unsigned col,
+                                              const float4& target)
+{
+    const int sid = a.sy.S == 1 ? 0 : find_system(a.sy.pbase, a.sy.S, __float_as_uint(target.w));
+    const SysDesc& d = a.sy.sys[sid];
+    const Grid& g = d.g;
+    const float4 t[1] = {target};
+    const int cx[1] = {axis_cell(target.x, g.lo[0], g.inv_w[0], g.n[0])};
+    const int cy = axis_cell(target.y, g.lo[1], g.inv_w[1], g.n[1]);
+    const int cz = axis_cell(target.z, g.lo[2], g.inv_w[2], g.n[2]);
+    int nw = 0;
+    {
+        uint32_t ulo[9], uhi[9];
+#pragma unroll
+        for (int rr = 0; rr < 9; ++rr) {
+            ulo[rr] = 0xffffffffu;
+            uhi[rr] = 0u;
+        }
+        group_windows_direct<DENSE, 1>(a, d, t, cx, cy, cz, ulo, uhi);
+#pragma unroll
+        for (int rr = 0; rr < 9; ++rr)
+            if (uhi[rr] > ulo[rr] && PI_BOUNDS(a.ctrl, 2 * nw + 1, 18, CS_DIRECT_WIN)) {
+                win[2 * nw][col] = ulo[rr];
+                win[2 * nw + 1][col] = uhi[rr];
+                ++nw;
+            }
+    }
+    // nw >= 1: the window of the target's own row holds it
+#ifdef PI_CHECK
+    if (!PI_BOUNDS(a.ctrl, nw > 0 ? 0 : 1, 1, CS_DIRECT_WIN)) return;
+#endif
+    const float rc2 = d.rc2;
+    const KParams kp = kparams(a, sid);
+    const float2 ks = make_float2(kp.t, kp.t);
+    Sums<Acc, KERNEL> r;
+    float n = 0.f;
+    const uint32_t wb = smem_addr(&win[0][col]);
+    constexpr uint32_t WSTEP = (uint32_t)WT * 8u;  // one window = two rows of win
+    const uint32_t we = wb + (uint32_t)nw * WSTEP;
+    uint32_t wa = wb;
+    uint32_t c = lds_u32(wa), ce = lds_u32(wa + WT * 4u);
+    do {
+        if (!PI_BOUNDS(a.ctrl, (uint64_t)c + 3u, a.np, CS_DIRECT_SRC)) break;
+        const float4* q = a.P + c;
+        const float4 s0 = __ldg(q), s1 = __ldg(q + 1), s2 = __ldg(q + 2), s3 = __ldg(q + 3);
+        cand_sources<KERNEL>(s0, s1, target, rc2, ks, kp, r, n);
+        cand_sources<KERNEL>(s2, s3, target, rc2, ks, kp, r, n);
+        c += 4u;
+        const bool sw = c >= ce;
+        wa += sw ? WSTEP : 0u;
+        const uint32_t cn = lds_u32(wa), cen = lds_u32(wa + WT * 4u);
+        c = sw ? cn : c;
+        ce = sw ? cen : ce;
+    } while (wa < we);
+    r.n = (uint32_t)n;  // exact: at most 2^24 neighbours
+    store_out(a, __float_as_uint(target.w), r);
+}
+
+// The target with exact window bounds in dense cells, out of line so that
+// the common path keeps its code and registers.
+template <class Acc, int KERNEL>
+__device__ __noinline__ void direct_single_dense(const InteractArgs& a, uint32_t (*win)[DIRECT_THREADS], unsigned col,
+                                                 const float4& target)
+{
+    direct_single<DIRECT_THREADS, true, Acc, KERNEL>(a, win, col, target);
+}
+
+// P slot p per thread.  Against the pair form each target is evaluated over
+// its own windows only (about 120 candidates at 8 per cell against 146, with
+// the padding of four-source trips) but every source read feeds one target
+// instead of two, and the sums are scalar.  What bounds a small launch is
+// the latency of one thread's chain of trips, which one target halves; what
+// bounds a large one of the costly forms is arithmetic per evaluation.  The
+// launch rule and its figures are at one_target_form (pi_api.cu).
+template <class Acc, int KERNEL>
+__global__ void __launch_bounds__(DIRECT_THREADS, 6) k_interact_direct1(InteractArgs a)
+{
+    __shared__ uint32_t win[20][DIRECT_THREADS];  // 9 windows (lo, hi) + one spare read after the last
+    pdl_trigger();
+    pdl_wait();  // the binning (or the previous interaction) has completed
+    // keep the work counters of the tiled launches in step (see k_interact_tiled)
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.ctrl->work[(a.seq + 1u) & 1u] = 0u;
+    const uint32_t k = blockIdx.x * DIRECT_THREADS + threadIdx.x;
+    // the control words and the target in flight together
+    const uint32_t err = load_error(a.ctrl);
+    const uint32_t mpc = *((volatile const uint32_t*)&a.ctrl->max_per_cell);
+    if (k >= a.np) return;
+    const float4 t = __ldg(a.P + k);
+    if (err || __float_as_uint(t.w) == 0xffffffffu) return;
+    if (mpc > DENSE_CELL)
+        direct_single_dense<Acc, KERNEL>(a, win, threadIdx.x, t);
+    else
+        direct_single<DIRECT_THREADS, false, Acc, KERNEL>(a, win, threadIdx.x, t);
+}
+
 // Resident CTAs per SM the four-target direct kernel's registers are capped
 // for (the plain kernels: 5, about 100 registers; the others uncapped).
 template <class Acc, int KERNEL>
@@ -1761,6 +1897,10 @@ void launch_direct4_one(const InteractArgs& a, cudaStream_t s)
 template <class Acc, int KERNEL>
 void launch_direct_one(const InteractArgs& a, cudaStream_t s)
 {
+    if (a.one_target && !a.ranges && !a.count_evals) {
+        (void)launch_dependent(k_interact_direct1<Acc, KERNEL>, dim3(direct_grid(a, 1)), dim3(DIRECT_THREADS), 0, s, a);
+        return;
+    }
     // an error is left for cudaGetLastError
     if constexpr (counted_form<Acc, KERNEL>()) {
         if (a.count_evals) {

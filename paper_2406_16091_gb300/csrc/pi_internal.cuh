@@ -487,6 +487,7 @@ struct InteractArgs {
     int nranges;
     unsigned range_blocks;
     int count_evals;        // direct kernels: add their evaluations to ctrl->evals
+    int one_target;         // shape 5: one target per thread instead of two (whole launches, not counting)
 };
 
 // Each adds the number of kernels it launched to *launches.
