@@ -693,8 +693,7 @@ pi_status pi_batch_bin(pi_ctx* ctx, const float* x, const float* y, const float*
                            ctx->S + 1, s));
     ctx->launches += 1;
     if (nn > 0) {
-        PI_TRY(pi::launch_hist(x, y, z, nn, sy, ctx->counts, ctx->cell, ctx->rank, ctx->ctrl,
-                               ctx->num_sms, s));
+        PI_TRY(pi::launch_hist(x, y, z, nn, sy, ctx->counts, ctx->cell, ctx->rank, ctx->ctrl, s));
         ctx->launches += 1;
     }
     PI_TRY(pi::launch_scan(ctx->counts, C, ctx->offsets, ctx->scan_status, ctx->ctrl, ctx->epoch,

@@ -407,7 +407,7 @@ cudaError_t launch_zero(uint32_t* p, size_t n_words, uint32_t* pbase, const uint
                         cudaStream_t s);
 cudaError_t launch_hist(const float* x, const float* y, const float* z, uint32_t n,
                         const Systems& sy, uint32_t* counts, uint32_t* cell, uint32_t* rank,
-                        Ctrl* ctrl, int num_sms, cudaStream_t s);
+                        Ctrl* ctrl, cudaStream_t s);
 // track_max: also record the largest count in Ctrl::max_per_cell (M_C);
 // ticket_slot: 0 takes the tiles from Ctrl::ticket, 1..3 from
 // Ctrl::tickets[slot - 1] (each scan of a step needs its own, cleared by
