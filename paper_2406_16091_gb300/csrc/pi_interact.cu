@@ -1484,6 +1484,7 @@ __device__ __forceinline__ uint32_t direct_group(const InteractArgs& a, const Sy
                 ++nw;
             }
     }
+    if constexpr (WIDE) win[2 * nw][col] = nw > 0 ? win[0][col] : 0u;
     // nw >= 1: the window of the first target's own row holds it
 #ifdef PI_CHECK
     // (a debug build whose checks dropped every window has nothing to read)
@@ -1502,35 +1503,58 @@ __device__ __forceinline__ uint32_t direct_group(const InteractArgs& a, const Sy
     const uint32_t we = wb + (uint32_t)nw * WSTEP;
     uint32_t wa = wb;
     uint32_t c = lds_u32(wa), ce = lds_u32(wa + WT * 4u);
-    do {
-        if (!PI_BOUNDS(a.ctrl, (uint64_t)c + 3u, a.np, CS_DIRECT_SRC) ||
-            !PI_BOUNDS(a.ctrl, WIDE ? c & 1u : 0u, 1u, CS_DIRECT_SRC))
-            break;
-        const float4* q = a.P + c;
-        float4 s0, s1, s2, s3;
-        if constexpr (WIDE) {
-            ldg_pair(q, s0, s1);
-            ldg_pair(q + 2, s2, s3);
-        } else {
-            s0 = __ldg(q);
-            s1 = __ldg(q + 1);
-            s2 = __ldg(q + 2);
-            s3 = __ldg(q + 3);
-        }
+    // two sources against every target of the group
+    auto eval = [&](const float4& u, const float4& v) {
 #pragma unroll
         for (int h = 0; h < G / 2; ++h) {
-            ps[h].cand(s0, t[2 * h], t[2 * h + 1], rc2, ks, kp);
-            ps[h].cand(s1, t[2 * h], t[2 * h + 1], rc2, ks, kp);
-            ps[h].cand(s2, t[2 * h], t[2 * h + 1], rc2, ks, kp);
-            ps[h].cand(s3, t[2 * h], t[2 * h + 1], rc2, ks, kp);
+            ps[h].cand(u, t[2 * h], t[2 * h + 1], rc2, ks, kp);
+            ps[h].cand(v, t[2 * h], t[2 * h + 1], rc2, ks, kp);
         }
+    };
+    // the next trip: c + 4, or the next window's start
+    auto advance = [&]() {
         c += 4u;
         const bool sw = c >= ce;
         wa += sw ? WSTEP : 0u;
         const uint32_t cn = lds_u32(wa), cen = lds_u32(wa + WT * 4u);
         c = sw ? cn : c;
         ce = sw ? cen : ce;
-    } while (wa < we);
+    };
+    if constexpr (WIDE) {
+        // Half a trip ahead: while two sources are evaluated the next two are
+        // on their way, in the registers a whole trip takes anyway.  With
+        // four targets that is 8 evaluations, enough to cover a load from L1
+        // and, over the SM's 20 warps, most of one from L2.  (Medians with
+        // the trip loaded whole / half ahead: 8 per cell 239.6 / 235.5 us at
+        // 2 M and 1810 / 1767 at 16.8 M, 16 per cell 350 / 346, 32 per cell
+        // 641 / 641.  With two targets per thread it was slower, clustered
+        // 1264 / 1280, and so was a step of two sources, 8 per cell 239.6.)
+        // The last trip prefetches the first window's start again: the spare
+        // window read after the last one holds it.
+        float4 s0, s1, s2, s3;
+        if (!PI_BOUNDS(a.ctrl, (uint64_t)c + 1u, a.np, CS_DIRECT_SRC)) c = 0u;
+        ldg_pair(a.P + c, s0, s1);
+        do {
+            if (!PI_BOUNDS(a.ctrl, (uint64_t)c + 3u, a.np, CS_DIRECT_SRC) ||
+                !PI_BOUNDS(a.ctrl, c & 1u, 1u, CS_DIRECT_SRC))
+                break;
+            ldg_pair(a.P + c + 2u, s2, s3);
+            eval(s0, s1);
+            advance();
+            if (!PI_BOUNDS(a.ctrl, (uint64_t)c + 3u, a.np, CS_DIRECT_SRC)) break;
+            ldg_pair(a.P + c, s0, s1);
+            eval(s2, s3);
+        } while (wa < we);
+    } else {
+        do {
+            if (!PI_BOUNDS(a.ctrl, (uint64_t)c + 3u, a.np, CS_DIRECT_SRC)) break;
+            const float4* q = a.P + c;
+            const float4 s0 = __ldg(q), s1 = __ldg(q + 1), s2 = __ldg(q + 2), s3 = __ldg(q + 3);
+            eval(s0, s1);
+            eval(s2, s3);
+            advance();
+        } while (wa < we);
+    }
 #pragma unroll
     for (int k = 0; k < G; ++k) ps[k / 2].to(r[k], (k & 1) != 0);
     return slots;
