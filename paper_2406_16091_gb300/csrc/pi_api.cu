@@ -71,7 +71,7 @@ struct pi_ctx {
     std::vector<float> kscale_h;    // [2S] per-system kernel scales last written to d_kscale
     int binned;                     // a pi_bin has been enqueued since the last failure
     uint32_t epoch;                 // scan launch epoch
-    uint64_t launches;              // kernels launched
+    mutable uint64_t launches;      // kernels launched
     uint32_t tiled_seq;             // launches of the tiled interaction kernel
     int algo;
     int precision;
@@ -525,14 +525,27 @@ pi_status pi_copy_binned(const pi_ctx* ctx, uint32_t* counts, uint32_t* offsets,
     if (ds.err != cudaSuccess) return cuda_fail(ds.err, "pi_copy_binned: set device");
     cudaStream_t s = (cudaStream_t)stream;
     const size_t C = (size_t)ctx->C, n = (size_t)ctx->n;
-    const cudaMemcpyKind k = cudaMemcpyDeviceToDevice;
-    if (counts) PI_TRY(cudaMemcpyAsync(counts, ctx->counts, C * 4, k, s));
-    if (offsets) PI_TRY(cudaMemcpyAsync(offsets, ctx->offsets, (C + 1) * 4, k, s));
-    if (n > 0) {
-        if (perm) PI_TRY(cudaMemcpyAsync(perm, ctx->perm, n * 4, k, s));
-        if (sx) PI_TRY(cudaMemcpyAsync(sx, ctx->sx, n * 4, k, s));
-        if (sy) PI_TRY(cudaMemcpyAsync(sy, ctx->sy, n * 4, k, s));
-        if (sz) PI_TRY(cudaMemcpyAsync(sz, ctx->sz, n * 4, k, s));
+    const void* src[6] = {ctx->counts, ctx->offsets, ctx->perm, ctx->sx, ctx->sy, ctx->sz};
+    void* dst[6] = {counts, offsets, perm, sx, sy, sz};
+    const size_t words[6] = {C, C + 1, n, n, n, n};
+    // one dependent launch for all the arrays; a destination that is not
+    // word-aligned goes by a memory copy (step with one array copied after
+    // it, by a memory copy / by this launch: 26.9 / 25.7 us at 1,531
+    // particles, 35.1 / 33.9 at 32,768, 441 / 437 for 64 systems)
+    pi::CopyArgs c{};
+    for (int k = 0; k < 6; ++k) {
+        if (!dst[k] || words[k] == 0) continue;
+        if ((uintptr_t)dst[k] % 4 != 0) {
+            PI_TRY(cudaMemcpyAsync(dst[k], src[k], words[k] * 4, cudaMemcpyDeviceToDevice, s));
+            continue;
+        }
+        c.src[c.count] = (const uint32_t*)src[k];
+        c.dst[c.count] = (uint32_t*)dst[k];
+        c.words[c.count++] = words[k];
+    }
+    if (c.count > 0) {
+        PI_TRY(pi::launch_copy_words(c, s));
+        ctx->launches += 1;
     }
     return PI_OK;
 }

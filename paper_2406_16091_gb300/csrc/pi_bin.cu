@@ -651,6 +651,37 @@ cudaError_t launch_write_words(uint32_t* dst, const uint32_t* vals, size_t count
     return cudaSuccess;
 }
 
+namespace {
+// The arrays of one CopyArgs, blockIdx.y choosing the array.  The sources are
+// 256-byte aligned (the arena's); a destination that is not 16-byte aligned
+// is written word by word.
+__global__ void __launch_bounds__(256) k_copy_words(CopyArgs c)
+{
+    pdl_wait();
+    const uint32_t* __restrict__ src = c.src[blockIdx.y];
+    uint32_t* __restrict__ dst = c.dst[blockIdx.y];
+    const size_t n = c.words[blockIdx.y], tid = (size_t)blockIdx.x * blockDim.x + threadIdx.x,
+                 threads = (size_t)gridDim.x * blockDim.x;
+    size_t done = 0;
+    if (((uintptr_t)dst & 15u) == 0) {
+        const size_t n4 = n / 4;
+        for (size_t k = tid; k < n4; k += threads)
+            reinterpret_cast<uint4*>(dst)[k] = reinterpret_cast<const uint4*>(src)[k];
+        done = 4 * n4;
+    }
+    for (size_t k = done + tid; k < n; k += threads) dst[k] = src[k];
+}
+}  // namespace
+
+cudaError_t launch_copy_words(const CopyArgs& c, cudaStream_t s)
+{
+    size_t most = 0;
+    for (int k = 0; k < c.count; ++k) most = std::max(most, c.words[k]);
+    // four 16-byte groups per thread at the most
+    const size_t blocks = std::min<size_t>(std::max<size_t>(1, (most + 4095) / 4096), 16384);
+    return launch_dependent(k_copy_words, dim3((unsigned)blocks, (unsigned)c.count), dim3(256), 0, s, c);
+}
+
 cudaError_t launch_set_kscale(float* kscale, const float* vals, int count, cudaStream_t s)
 {
     if (count < 0 || count > 2 * MAX_SYSTEMS) return cudaErrorInvalidValue;

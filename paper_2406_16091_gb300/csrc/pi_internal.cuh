@@ -440,6 +440,16 @@ cudaError_t launch_set_system(SysDesc* sys, uint32_t* cbase, uint32_t* wbase, ui
 // may be captured in a CUDA graph); vals is read before the call returns.
 cudaError_t launch_write_words(uint32_t* dst, const uint32_t* vals, size_t count, cudaStream_t s);
 
+// Up to six device arrays of 32-bit words (sources in the arena,
+// destinations 4-byte aligned) copied by one dependent launch.
+struct CopyArgs {
+    const uint32_t* src[6];
+    uint32_t* dst[6];
+    size_t words[6];
+    int count;
+};
+cudaError_t launch_copy_words(const CopyArgs& c, cudaStream_t s);
+
 // Per-system scales of the interaction kernel, written from launch
 // parameters (vals[i] for i < count, count <= 2 MAX_SYSTEMS) into kscale.
 cudaError_t launch_set_kscale(float* kscale, const float* vals, int count, cudaStream_t s);
