@@ -49,7 +49,6 @@ __global__ void __launch_bounds__(CHUNK_THREADS, 2) k_bucket_count(const float* 
                                                                 int vec)
 {
     extern __shared__ uint32_t hist[];
-    pdl_trigger();
     for (uint32_t b = threadIdx.x; b < plan.B; b += CHUNK_THREADS) hist[b] = 0u;
     __syncthreads();
     pdl_wait();  // the particle bases and the control block are k_zero's
@@ -87,7 +86,6 @@ __global__ void __launch_bounds__(CHUNK_THREADS, 2) k_bucket_scatter(const float
                                                                   int vec)
 {
     extern __shared__ uint32_t cur[];
-    pdl_trigger();
     pdl_wait();
     if (cta_error(ctrl)) return;
     const uint32_t k = blockIdx.x;
@@ -154,7 +152,6 @@ __global__ void __launch_bounds__(CELL_THREADS) k_bucket_cells(
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     CellSmem& sm = *reinterpret_cast<CellSmem*>(smem_raw);
-    pdl_trigger();
     pdl_wait();
     if (cta_error(ctrl)) return;
     const unsigned tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
@@ -339,7 +336,6 @@ __global__ void __launch_bounds__(256) k_bucket_big(const float4* __restrict__ r
                                                     float4* __restrict__ P, uint2* __restrict__ xbins,
                                                     const uint2* __restrict__ ovf_list, Ctrl* __restrict__ ctrl)
 {
-    pdl_trigger();
     pdl_wait();
     if (cta_error(ctrl)) return;
     const unsigned long long o = *((volatile const unsigned long long*)&ctrl->ovf);

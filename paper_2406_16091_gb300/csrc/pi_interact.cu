@@ -46,9 +46,9 @@
 //   k_interact_ws      the same chunks with a producer warp that stages them
 //                      for consumer warps (warp specialisation).
 // All of them sum each target's terms in the order of its own windows, so
-// their outputs are bitwise equal.  Every one is a programmatic dependent
-// launch: it may start while the binning's last kernel (or the previous
-// interaction) drains, and waits for it before reading anything of the step.
+// their outputs are bitwise equal.  Every one is a dependent launch: it waits
+// for the binning's last kernel (or the previous interaction) before reading
+// anything of the step.
 #include <type_traits>
 
 #include "pi_internal.cuh"
@@ -229,7 +229,6 @@ __device__ __forceinline__ void store_out(const InteractArgs& a, uint32_t slot, 
 template <class Acc, int KERNEL>
 __global__ void __launch_bounds__(128) k_interact_ppnl(InteractArgs a)
 {
-    pdl_trigger();
     pdl_wait();
     if (cta_error(a.ctrl)) return;
     const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -979,7 +978,6 @@ __global__ void __launch_bounds__(T::NT, T::MINB) k_interact_tiled(InteractArgs 
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Smem<T>& sm = *reinterpret_cast<Smem<T>*>(smem_raw);
 
-    pdl_trigger();
     pdl_wait();
     if (blockIdx.x == 0 && threadIdx.x == 0) a.ctrl->work[(a.seq + 1u) & 1u] = 0u;
     const unsigned tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
@@ -1296,7 +1294,6 @@ __global__ void __launch_bounds__(T::THREADS, T::MINB) k_interact_ws(InteractArg
     extern __shared__ __align__(16) unsigned char smem_raw[];
     WsSmem<T>& sm = *reinterpret_cast<WsSmem<T>*>(smem_raw);
     const unsigned tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
-    pdl_trigger();
     pdl_wait();
     if (tid == 0) {
         if (blockIdx.x == 0) a.ctrl->work[(a.seq + 1u) & 1u] = 0u;
@@ -1671,7 +1668,6 @@ __global__ void __launch_bounds__(DIRECT_THREADS, (direct_min_blocks<Acc, KERNEL
     k_interact_direct(InteractArgs a)
 {
     __shared__ uint32_t win[20][DIRECT_THREADS];  // 9 windows (lo, hi) + one spare read after the last
-    pdl_trigger();
     pdl_wait();  // the binning (or the previous interaction) has completed
     // keep the work counters of the tiled launches in step (see k_interact_tiled)
     if (blockIdx.x == 0 && threadIdx.x == 0) a.ctrl->work[(a.seq + 1u) & 1u] = 0u;
@@ -1798,7 +1794,6 @@ template <class Acc, int KERNEL>
 __global__ void __launch_bounds__(DIRECT_THREADS, 6) k_interact_direct1(InteractArgs a)
 {
     __shared__ uint32_t win[20][DIRECT_THREADS];  // 9 windows (lo, hi) + one spare read after the last
-    pdl_trigger();
     pdl_wait();  // the binning (or the previous interaction) has completed
     // keep the work counters of the tiled launches in step (see k_interact_tiled)
     if (blockIdx.x == 0 && threadIdx.x == 0) a.ctrl->work[(a.seq + 1u) & 1u] = 0u;
@@ -1835,7 +1830,6 @@ __global__ void __launch_bounds__(DIRECT_THREADS, (direct4_min_blocks<Acc, KERNE
     k_interact_direct4(InteractArgs a)
 {
     __shared__ uint32_t win[20][DIRECT_THREADS];  // 9 windows (lo, hi) + one spare read after the last
-    pdl_trigger();
     pdl_wait();  // the binning (or the previous interaction) has completed
     // keep the work counters of the tiled launches in step (see k_interact_tiled)
     if (blockIdx.x == 0 && threadIdx.x == 0) a.ctrl->work[(a.seq + 1u) & 1u] = 0u;

@@ -281,16 +281,24 @@ __device__ __forceinline__ uint64_t global_ns()
     return t;
 }
 
-// Programmatic dependent launch.  A kernel started by launch_dependent may
-// begin while the kernel before it in the stream is still running (once
-// every block of that kernel has called pdl_trigger or exited); pdl_wait
-// then blocks until that kernel has completed and its writes are visible.
-// The default binning kernels never trigger (see pi_bin.cu): their
-// successor's blocks are placed as their own exit, evenly over the SMs.
-// Whatever a kernel reads or writes of the step's state comes after its
-// pdl_wait.  For a kernel launched the ordinary way both are no-ops.
+// Programmatic dependent launch.  A kernel started by launch_dependent is
+// launched while the kernel before it in the stream still runs; its blocks
+// are released as that kernel's last ones exit, and pdl_wait then blocks
+// until that kernel has completed and its writes are visible.  Whatever a
+// kernel reads or writes of the step's state comes after its pdl_wait.  For
+// a kernel launched the ordinary way it is a no-op.
+//
+// No kernel releases its successor early (griddepcontrol.launch_dependents):
+// released on entry, the successor's blocks were placed while the kernel
+// still held its SMs, so a grid of less than a wave piled up on the SMs that
+// happened to be free, and all they could do there was wait.  The
+// interaction of 32,768 particles (128 CTAs) then took 38 instead of 20 us.
+// Measured, step of pi_bin + pi_interact with the release on entry / at
+// exit: 57 / 36 us at 32,768 particles, 60 / 38 at 65,536, 56 / 42 at
+// 131,072, 328 / 324 at 2.1 M; bucketed binning 67 / 42 at 32,768 and 345 /
+// 334 at 2.1 M, radix 70 / 52 and 434 / 421; four interactions in a row at
+// 262,147 particles 33.7 / 31.1 each.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <class... KArgs, class... Args>
 inline cudaError_t launch_dependent(void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,

@@ -58,7 +58,6 @@ __global__ void __launch_bounds__(RADIX_THREADS) k_radix_keys(const float* __res
                                                               int vec)
 {
     extern __shared__ uint32_t hist[];
-    pdl_trigger();
     for (uint32_t b = threadIdx.x; b < plan.bins; b += RADIX_THREADS) hist[b] = 0u;
     __syncthreads();
     pdl_wait();  // the particle bases and the control block are k_zero's
@@ -94,7 +93,6 @@ __global__ void __launch_bounds__(RADIX_THREADS) k_radix_count(const uint32_t* _
                                                                uint32_t* __restrict__ mat, Ctrl* __restrict__ ctrl)
 {
     extern __shared__ uint32_t hist[];
-    pdl_trigger();
     for (uint32_t b = threadIdx.x; b < plan.bins; b += RADIX_THREADS) hist[b] = 0u;
     __syncthreads();
     pdl_wait();
@@ -123,7 +121,6 @@ __global__ void __launch_bounds__(RADIX_THREADS) k_radix_scatter(const uint32_t*
     const uint32_t bins = plan.bins, mask = bins - 1u;
     uint32_t* cnt = sm;                           // [warp][bins]
     uint32_t* gb = sm + RADIX_WARPS * bins;       // [bins]
-    pdl_trigger();
     const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     for (uint32_t b = lane; b < bins; b += 32) cnt[warp * bins + b] = 0u;
     pdl_wait();
@@ -190,7 +187,6 @@ __global__ void __launch_bounds__(256) k_radix_gather(const uint32_t* __restrict
                                                       float* __restrict__ sx, float* __restrict__ sy_out,
                                                       float* __restrict__ sz, Ctrl* __restrict__ ctrl)
 {
-    pdl_trigger();
     pdl_wait();
     if (cta_error(ctrl)) return;
     bool bad = false;
@@ -218,7 +214,6 @@ __global__ void __launch_bounds__(256) k_radix_rank(const uint32_t* __restrict__
                                                     float4* __restrict__ P, uint2* __restrict__ xbins,
                                                     Ctrl* __restrict__ ctrl)
 {
-    pdl_trigger();
     pdl_wait();
     if (cta_error(ctrl)) return;
     const uint32_t rows = __ldg(sy.rbase + sy.S);
