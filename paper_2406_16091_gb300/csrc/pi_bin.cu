@@ -17,14 +17,7 @@
 //
 // All kernels are HBM- or L2-bound integer work; none uses tensor cores.
 //
-// Every kernel after k_zero is a dependent launch (see launch_dependent), but
-// none of them calls pdl_trigger: the next kernel's blocks are released as
-// this one's exit.  Triggered on entry, they were placed while this kernel
-// still held its SMs, so a grid of less than a wave piled up on the SMs that
-// happened to be free: the interaction of 32,768 particles (128 CTAs) then
-// took 38 instead of 20 us.  Measured, step of pi_bin + pi_interact with the
-// trigger on entry / at exit: 57 / 36 us at 32,768 particles, 60 / 38 at
-// 65,536, 56 / 42 at 131,072, 328 / 324 at 2.1 M (binning 93 / 89).
+// Every kernel is a dependent launch (see launch_dependent).
 #include <algorithm>
 #include <mutex>
 
@@ -39,6 +32,11 @@ constexpr unsigned FULL = 0xffffffffu;
 template <int NB>
 __global__ void k_zero(ZeroArgs<NB> z)
 {
+    // the previous step's kernels still read what this one clears; nothing
+    // of this step starts before its blocks have exited, so whatever ran
+    // before it in the stream (the positions' producer too) is complete by
+    // then
+    pdl_wait();
     size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     size_t stride = (size_t)gridDim.x * blockDim.x;
     uint4* p4 = reinterpret_cast<uint4*>(z.p);
@@ -97,7 +95,7 @@ __global__ void __launch_bounds__(256) k_hist(const float* __restrict__ x,
                 pz[j] = valid[j] ? z[i] : 0.f;
             }
         }
-        // the positions are the caller's input, written before k_zero started;
+        // the positions are the caller's input, complete before k_zero ended;
         // the particle bases and the counts are k_zero's
         pdl_wait();
         int s = (sy.S == 1 || grp >= groups) ? 0 : find_system(sy.pbase, sy.S, i0);
@@ -530,8 +528,7 @@ cudaError_t launch_zero_nb(uint32_t* p, size_t n_words, uint32_t* pbase, const u
     for (int k = 0; k < nb; ++k) z.vals[k] = vals[k];
     int blocks = (int)((n_words / 4 + 255) / 256);
     blocks = blocks < 1 ? 1 : (blocks > 1184 ? 1184 : blocks);
-    k_zero<NB><<<blocks, 256, 0, s>>>(z);
-    return cudaGetLastError();
+    return launch_dependent(k_zero<NB>, dim3((unsigned)blocks), dim3(256), 0, s, z);
 }
 
 cudaError_t launch_zero(uint32_t* p, size_t n_words, uint32_t* pbase, const uint32_t* vals, int nb,
