@@ -185,7 +185,7 @@ float kernel_scale(int kernel, float h)
     const double hd = (double)h;
     switch (kernel) {
         case PI_KERNEL_LJ:
-        case PI_KERNEL_HIGHFLOP: return h * h;  // sigma^2 in FP32
+        case PI_KERNEL_HIGHFLOP: return (float)std::fmin(1.0 / (hd * hd), (double)FLT_MAX);  // 1 / sigma^2, finite
         case PI_KERNEL_LOWFLOP: return 0.f;
         default: return (float)(-1.4426950408889634 / (hd * hd));  // -log2(e) / h^2
     }
@@ -203,15 +203,17 @@ float kernel_scale_lo(int kernel, float h)
 // Whether the scale of h is usable: finite for the Gaussian (below about
 // h = 6.5e-20 it overflows FP32, and 0 * -inf would turn the term of two
 // coincident particles into NaN), finite and non-zero for Lennard-Jones
-// (sigma^2 = h^2 must neither overflow nor flush to zero).
+// (sigma^2 = h^2 in FP32 must neither overflow nor flush to zero).
 bool scale_ok(int kernel, float h)
 {
-    const float t = kernel_scale(kernel, h);
     switch (kernel) {
         case PI_KERNEL_LJ:
-        case PI_KERNEL_HIGHFLOP: return std::isfinite(t) && t > 0.f;
+        case PI_KERNEL_HIGHFLOP: {
+            const float sigma2 = h * h;
+            return std::isfinite(sigma2) && sigma2 > 0.f;
+        }
         case PI_KERNEL_LOWFLOP: return true;
-        default: return std::isfinite(t);
+        default: return std::isfinite(kernel_scale(kernel, h));
     }
 }
 
