@@ -805,11 +805,11 @@ pi_status launch_plan(pi_ctx* ctx, pi::InteractArgs a, bool kahan, cudaStream_t 
 // of two.  Medians of the interaction in us, two targets / one (particles,
 // mean per cell):
 //   - few particles: one thread's chain of trips sets the time, and one
-//     target halves it, up to about 256 threads per SM of the plain and the
-//     compensated sums (Gaussian: 1,531 at 6 18.4 / 14.4, 10,000 at 8 22.5 /
-//     16.4, 32,768 at 8 20.5 / 18.4, 65,536 at 8 22.5 / 24.6) and 1024 of
-//     the costlier kernels (Lennard-Jones at 8: 30,000 34.8 / 24.6, 131,072
-//     45.1 / 38.9, 262,144 61.4 / 65.5);
+//     target halves it, up to about 256 threads per SM (Gaussian: 1,531 at 6
+//     18.4 / 14.4, 10,000 at 8 22.5 / 16.4, 32,768 at 8 20.5 / 18.4, 65,536
+//     at 8 22.5 / 24.6; Lennard-Jones: 30,000 clustered 41.0 / 30.7, 60,000
+//     at 8 24 / 22.5, 131,072 at 8 34.8 / 34.8, 100,000 dense clusters 207 /
+//     299);
 //   - the 168-FLOP kernel spends most on each evaluation, and one target
 //     has fewer of them: 465 / 375 and 975 / 922 (2 M at 2 and 8), dense
 //     clusters 2540 / 2132 (300,000 at 16);
@@ -820,10 +820,8 @@ pi_status launch_plan(pi_ctx* ctx, pi::InteractArgs a, bool kahan, cudaStream_t 
 //     317 (100,000 at 16).
 bool one_target_form(const pi_ctx* ctx, int kernel)
 {
-    const bool kahan = ctx->precision == PI_PREC_KAHAN;
-    const bool plain = !kahan && (kernel == pi::KERNEL_GAUSSIAN || kernel == pi::KERNEL_LOWFLOP);
-    if (ctx->n <= (int64_t)ctx->num_sms * (plain || kahan ? 256 : 1024)) return true;
-    if (kahan) return ctx->n < 4 * ctx->C;
+    if (ctx->n <= (int64_t)ctx->num_sms * 256) return true;
+    if (ctx->precision == PI_PREC_KAHAN) return ctx->n < 4 * ctx->C;
     if (kernel == pi::KERNEL_GAUSSIAN_FINE) return ctx->n < 16 * ctx->C;
     return kernel == pi::KERNEL_HIGHFLOP;
 }

@@ -13,7 +13,7 @@ from gpu_harness import check_interaction, oracle_run, run_gpu
 
 pytestmark = pytest.mark.gpu
 
-SMS = 152  # of one GB300; the sizes below lie on both sides of the lines there
+SMS = 152  # of one GB300; the sizes below lie on both sides of the line there
 
 
 def _uniform(n, ppc, seed=31):
@@ -37,7 +37,7 @@ CASES = {
     "dense": lambda: _dense(6001),
     "line_256": lambda: _uniform(SMS * 256, 3),
     "past_256": lambda: _uniform(SMS * 256 + 1, 5),
-    "past_1024": lambda: _uniform(SMS * 1024 + 1, 3),
+    "larger": lambda: _uniform(SMS * 1024 + 1, 3),
 }
 FORMS = [(B.PI_KERNEL_GAUSSIAN, B.PI_PREC_FP32, 2), (B.PI_KERNEL_GAUSSIAN, B.PI_PREC_KAHAN, 2),
          (B.PI_KERNEL_GAUSSIAN, B.PI_PREC_FP32, 8), (B.PI_KERNEL_LJ, B.PI_PREC_FP32, 2),
