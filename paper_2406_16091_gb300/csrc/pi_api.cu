@@ -814,16 +814,17 @@ pi_status launch_plan(pi_ctx* ctx, pi::InteractArgs a, bool kahan, cudaStream_t 
 //     has fewer of them: 465 / 375 and 975 / 922 (2 M at 2 and 8), dense
 //     clusters 2540 / 2132 (300,000 at 16);
 //   - the compensated exponent likewise below 16 per cell: 242 / 213, 473 /
-//     469 and 1436 / 1464 (2 M at 2, 8 and 32);
-//   - the compensated sums below 4 per cell: 211 / 203, 406 / 410 and 1221 /
-//     1251 (2 M at 2, 8 and 32), clustered 690 / 627 (1 M at 2) and 287 /
-//     317 (100,000 at 16).
+//     469 and 1436 / 1464 (2 M at 2, 8 and 32), with compensated sums 180 /
+//     162 (500,000 at 8);
+//   - the compensated sums below 6 per cell: 211 / 195, 270 / 258 and 336 /
+//     322 (2 M at 2, 4 and 6), clustered 618 / 584 (1 M at 2) and 881 / 997
+//     (300,000 at 16: cells of more than 255 take their exact windows).
 bool one_target_form(const pi_ctx* ctx, int kernel)
 {
     if (ctx->n <= (int64_t)ctx->num_sms * 256) return true;
-    if (ctx->precision == PI_PREC_KAHAN) return ctx->n < 4 * ctx->C;
+    if (kernel == pi::KERNEL_HIGHFLOP) return true;
     if (kernel == pi::KERNEL_GAUSSIAN_FINE) return ctx->n < 16 * ctx->C;
-    return kernel == pi::KERNEL_HIGHFLOP;
+    return ctx->precision == PI_PREC_KAHAN && ctx->n < 6 * ctx->C;
 }
 
 // Occupancy regimes of the per-system autotuning: mean particles per cell
