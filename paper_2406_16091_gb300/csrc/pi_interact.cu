@@ -1471,6 +1471,108 @@ __device__ __forceinline__ void group_windows_direct(const InteractArgs& a, cons
     }
 }
 
+// The same ranges with the lookups of three rows in flight together.  One row
+// after the other, each row's lookups wait for L2 before the next row's
+// start: nine round trips, 3 of the 9 us that a small interaction takes
+// whatever its work.  Medians in us, row by row / three rows at a time: 1,531
+// particles 12.7 / 10.7, 32,768 15.3 / 13.2 (one target per thread), 2 M at 1
+// per cell 148.4 / 139.2, at 2 127.4 / 121.2 (two), at 8 230.3 / 229.3
+// (four).  All nine rows at once spill (12.2 and 14.8), and the compensated
+// sums, short of registers, are slower with it (1 M clustered 584 / 598).
+template <int G>
+__device__ __forceinline__ void group_windows_flat(const InteractArgs& a, const SysDesc& d, const float4 (&t)[G],
+                                                   const int (&cx)[G], int cy, int cz, uint32_t (&ulo)[9],
+                                                   uint32_t (&uhi)[9])
+{
+    constexpr int ROWS = 3;
+    Faces f[G];
+    int cmin = cx[0], cmax = cx[0];
+#pragma unroll
+    for (int k = 0; k < G; ++k) {
+        f[k] = faces_of(d, t[k].y, t[k].z, cy, cz);
+        cmin = min(cmin, cx[k]);
+        cmax = max(cmax, cx[k]);
+    }
+    const float rcm2 = d.rc2 * 1.00002f;
+    const float xlo = d.g.lo[0], slack = d.slack, invs = d.g.inv_w[0] * (float)XSUB;
+    const int nx = d.g.n[0], ny = d.g.n[1], nz = d.g.n[2];
+    const int lo = XSUB * max(cmin - 1, 0);
+    const int hi = XSUB * (min(cmax + 1, nx - 1) + 1) - 1;
+#pragma unroll
+    for (int r0 = 0; r0 < 9; r0 += ROWS) {
+        uint32_t o0[ROWS], o1[ROWS], w0[ROWS];
+        uint2 w1[ROWS];
+        int b0[ROWS], b1[ROWS];
+        bool has[ROWS];
+#pragma unroll
+        for (int q = 0; q < ROWS; ++q) {
+            const int rr = r0 + q, dy = rr % 3 - 1, dz = rr / 3 - 1;
+            const int by = cy + dy, bz = cz + dz;
+            float xl = INFINITY, xu = -INFINITY;
+#pragma unroll
+            for (int k = 0; k < G; ++k) {
+                const float ey = dy < 0 ? f[k].y_lo : (dy > 0 ? f[k].y_hi : 0.f);
+                const float ez = dz < 0 ? f[k].z_lo : (dz > 0 ? f[k].z_hi : 0.f);
+                const float tw = rcm2 - fmaf(ey, ey, ez * ez);
+                const float tt = fmaxf(tw, 1e-30f);
+                const float w = tt * rsqrtf(tt) + slack;
+                xl = tw > 0.f ? fminf(xl, t[k].x - w) : xl;
+                xu = tw > 0.f ? fmaxf(xu, t[k].x + w) : xu;
+            }
+            has[q] = by >= 0 && by < ny && bz >= 0 && bz < nz && xl <= xu;
+            // (a row without a window looks its own row up and drops it)
+            const uint32_t row = has[q] ? (uint32_t)by + (uint32_t)ny * (uint32_t)bz
+                                        : (uint32_t)cy + (uint32_t)ny * (uint32_t)cz;
+            b0[q] = sub_bin(has[q] ? xl : t[0].x, xlo, invs, 0, lo, hi);
+            b1[q] = sub_bin(has[q] ? xu : t[0].x, xlo, invs, 0, lo, hi) + 1;
+            const uint32_t rb = d.cell_base + (uint32_t)nx * row;
+            uint32_t cell0 = rb + (uint32_t)(b0[q] >> 3), cell1 = rb + (uint32_t)(b1[q] >> 3);
+#ifdef PI_CHECK
+            const uint64_t c_all = __ldg(a.sy.cbase + a.sy.S);
+            if (!PI_BOUNDS(a.ctrl, cell0, c_all, CS_DIRECT_LOOKUP)) cell0 = 0u, has[q] = false;
+            if (!PI_BOUNDS(a.ctrl, cell1, c_all + 1u, CS_DIRECT_LOOKUP)) cell1 = 0u, has[q] = false;
+#endif
+            o0[q] = __ldg(a.offsets + cell0);
+            o1[q] = __ldg(a.offsets + cell1);
+            // the sub-bin words: of the lower bound the half it needs (a cell
+            // without sub-bin starts has zeros there, its start); of the
+            // upper bound both, for the flag.  (Past the last cell one word
+            // is allocated, read only with a sub-bin of 0 and then not used.)
+            w0[q] = __ldg(reinterpret_cast<const uint32_t*>(a.xbins + cell0) + ((b0[q] & 7) > 4 ? 1 : 0));
+            w1[q] = __ldg(a.xbins + cell1);
+        }
+#pragma unroll
+        for (int q = 0; q < ROWS; ++q) {
+            const int by = cy + (r0 + q) % 3 - 1, bz = cz + (r0 + q) / 3 - 1;
+            const uint32_t row = (uint32_t)by + (uint32_t)ny * (uint32_t)bz, pad = ROW_PADS * (d.row_base + row);
+            const int s0 = b0[q] & 7, s1 = b1[q] & 7;
+            uint32_t j = o0[q], je = o1[q];
+            if (s0 != 0) j += (w0[q] >> (8 * ((s0 - 1) & 3))) & 255u;
+            if (s1 != 0 && has[q]) {
+                if ((w1[q].y >> 24) & XBIN_COARSE)
+                    je = __ldg(a.offsets + d.cell_base + (uint32_t)nx * row + (uint32_t)(b1[q] >> 3) + 1u);
+                else
+                    je += ((s1 <= 4 ? w1[q].x : w1[q].y) >> (8 * ((s1 - 1) & 3))) & 255u;
+            }
+            if (has[q] && je > j) {
+                ulo[r0 + q] = j + pad;
+                uhi[r0 + q] = je + pad;
+            }
+        }
+    }
+}
+
+template <bool DENSE, int G, class Acc>
+__device__ __forceinline__ void group_windows(const InteractArgs& a, const SysDesc& d, const float4 (&t)[G],
+                                              const int (&cx)[G], int cy, int cz, uint32_t (&ulo)[9],
+                                              uint32_t (&uhi)[9])
+{
+    if constexpr (!DENSE && std::is_same<Acc, PlainAcc>::value)
+        group_windows_flat<G>(a, d, t, cx, cy, cz, ulo, uhi);
+    else
+        group_windows_direct<DENSE, G>(a, d, t, cx, cy, cz, ulo, uhi);
+}
+
 // A group of G targets (a target may repeat the one before it)
 // of one X-row of one system: per row the union of their windows goes to
 // column `col` of `win` (rows where all are empty dropped), and one loop walks
@@ -1500,7 +1602,7 @@ __device__ __forceinline__ uint32_t direct_group(const InteractArgs& a, const Sy
             ulo[rr] = 0xffffffffu;
             uhi[rr] = 0u;
         }
-        group_windows_direct<DENSE, G>(a, d, t, cx, cy, cz, ulo, uhi);
+        group_windows<DENSE, G, Acc>(a, d, t, cx, cy, cz, ulo, uhi);
 #pragma unroll
         for (int rr = 0; rr < 9; ++rr)
             if (uhi[rr] > ulo[rr] && PI_BOUNDS(a.ctrl, 2 * nw + 1, 18, CS_DIRECT_WIN)) {
@@ -1771,7 +1873,7 @@ __device__ __forceinline__ void direct_single(const InteractArgs& a, uint32_t (*
             ulo[rr] = 0xffffffffu;
             uhi[rr] = 0u;
         }
-        group_windows_direct<DENSE, 1>(a, d, t, cx, cy, cz, ulo, uhi);
+        group_windows<DENSE, 1, Acc>(a, d, t, cx, cy, cz, ulo, uhi);
 #pragma unroll
         for (int rr = 0; rr < 9; ++rr)
             if (uhi[rr] > ulo[rr] && PI_BOUNDS(a.ctrl, 2 * nw + 1, 18, CS_DIRECT_WIN)) {
