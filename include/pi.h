@@ -109,7 +109,9 @@ enum {
      * it. */
     PI_OPT_TILE = 6,
     /* Binning: PI_BIN_PER_PARTICLE (default) takes one global atomic and
-     * one 32-byte provisional record per particle; PI_BIN_BUCKETED counts
+     * one 32-byte provisional record per particle (a system of at most 4096
+     * particles in at most 4096 cells is counted, scanned and scattered by
+     * one block from shared memory); PI_BIN_BUCKETED counts
      * the particles per bucket of consecutive cells and ranks each bucket's
      * cells in shared memory, when the bucket-by-chunk count matrix fits the
      * context (up to about 8 M cells; the per-particle path otherwise);

@@ -700,6 +700,18 @@ pi_status pi_batch_bin(pi_ctx* ctx, const float* x, const float* y, const float*
         return PI_OK;
     }
 
+    // a small system: everything before the ranking in one block
+    if (ctx->S == 1 && nn > 0 && nn <= pi::SMALL_MAX && C <= pi::SMALL_MAX && !ctx->withhold_scan) {
+        PI_TRY(pi::launch_bin_small(x, y, z, nn, sy, C, ctx->pbase, ctx->counts, ctx->offsets, ctx->xbins, ctx->rec,
+                                    ctx->ctrl, s));
+        PI_TRY(pi::launch_stabilise(ctx->rec, nn, sy, ctx->offsets, ctx->perm, ctx->sx, ctx->sy, ctx->sz, ctx->P,
+                                    ctx->xbins, ctx->ctrl, ctx->num_sms, s));
+        ctx->launches += 2;
+        ctx->n = total;
+        ctx->binned = 1;
+        return PI_OK;
+    }
+
     // per particle: control block, counts and xbins are one contiguous
     // zeroed prefix of the
     // arena; the same launch writes this step's particle bases

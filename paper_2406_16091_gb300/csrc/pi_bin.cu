@@ -10,6 +10,7 @@
 //   k_scatter    a4, first half: each particle (and its position) to its
 //                provisional slot (the paper's atomic scatter, whose order
 //                inside a cell is arbitrary)
+//   k_bin_small  all of the above for a small system, in one block
 //   k_stabilise  a4, second half: rank each particle among its cell's members
 //                by input index, which makes the order stable; write the
 //                sorted positions, the row-padded x-ordered copy P that the
@@ -19,6 +20,7 @@
 //
 // Every kernel is a dependent launch (see launch_dependent).
 #include <algorithm>
+#include <cstddef>
 #include <mutex>
 
 #include "pi_internal.cuh"
@@ -486,6 +488,114 @@ __global__ void __launch_bounds__(256) k_stabilise(const Rec* __restrict__ rec, 
     if (bad) atomicOr(&ctrl->error, ERR_CAPACITY);
 }
 
+// ---- a1 - a4's first half of a small system in one launch -----------------------
+//
+// k_zero, k_hist, k_scan and k_scatter cost about 3 us each whatever their
+// work: a launch and the round trips of their atomics and scans through L2.
+// A small system runs their phases in one block instead, with the counts,
+// the ranks' atomics and the scan in shared memory, and the phases separated
+// by block barriers; k_stabilise then follows as ever, over all SMs (its
+// work grows with the cells' occupancy).  Bound by those barriers and by one
+// SM's stores, so only up to 4096 particles: a step of pi_bin, pi_interact
+// and a copy took, with the five kernels / with this, 22.9 / 18.0 us at 1,531
+// particles, 23.7 / 21.9 at 4,096, 8 per cell (and on the device alone 19.0 /
+// 16.0 and 20.6 / 19.6; at 8,192 it was slower, 24.6 / 28.9).
+__global__ void __launch_bounds__(SMALL_THREADS)
+    k_bin_small(const float* __restrict__ x, const float* __restrict__ y, const float* __restrict__ z, uint32_t n,
+                Systems sy, uint32_t C, uint32_t* __restrict__ pbase, uint32_t* __restrict__ counts,
+                uint32_t* __restrict__ offsets, uint2* __restrict__ xbins, Rec* __restrict__ rec,
+                Ctrl* __restrict__ ctrl)
+{
+    constexpr int PER = SMALL_MAX / SMALL_THREADS;  // particles, and cells of the scan, per thread
+    static_assert(PER % 4 == 0, "the scan takes its cells four at a time");
+    __shared__ __align__(16) uint32_t s_off[SMALL_MAX];  // the counts, then the offsets
+    __shared__ uint32_t s_warp[SMALL_THREADS / 32], s_max[SMALL_THREADS / 32];
+    const uint32_t tid = threadIdx.x;
+    const unsigned lane = tid & 31u, warp = tid >> 5;
+    const SysDesc& d = sy.sys[0];
+
+    for (uint32_t k = tid; k < SMALL_MAX; k += SMALL_THREADS) s_off[k] = 0u;
+    pdl_wait();
+    uint32_t c[PER], r[PER];
+    bool all_ok = true;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        const uint32_t i = tid + j * SMALL_THREADS;
+        bool ok = true;
+        c[j] = i < n ? cell_of(x[i], y[i], z[i], d.g, ok) : 0u;
+        all_ok &= ok;
+    }
+    // (a barrier too: the counts are clear)
+    const bool ok = __syncthreads_and(all_ok) != 0;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        const bool valid = tid + j * SMALL_THREADS < n && PI_BOUNDS(ctrl, c[j], C, CS_HIST_COUNTS);
+        r[j] = valid ? atomicAdd(&s_off[c[j]], 1u) : 0u;
+    }
+    __syncthreads();
+    uint32_t v[PER], run = 0, mx = 0;
+#pragma unroll
+    for (int q = 0; q < PER / 4; ++q) {
+        const uint4 u = reinterpret_cast<const uint4*>(s_off)[tid * (PER / 4) + q];
+        v[4 * q] = u.x; v[4 * q + 1] = u.y; v[4 * q + 2] = u.z; v[4 * q + 3] = u.w;
+        const uint32_t c0 = tid * PER + 4 * q;
+        // (the counts and the offsets are padded to whole groups of four)
+        if (c0 < C) reinterpret_cast<uint4*>(counts)[c0 / 4] = u;
+    }
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        const uint32_t t = v[k];
+        mx = max(mx, t);
+        v[k] = run;
+        run += t;
+    }
+    uint32_t incl = run;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(FULL, incl, o);
+        if (lane >= (unsigned)o) incl += t;
+    }
+    mx = __reduce_max_sync(FULL, mx);
+    if (lane == 31) s_warp[warp] = incl;
+    if (lane == 0) s_max[warp] = mx;
+    __syncthreads();
+    uint32_t base = incl - run, block_max = 0;
+#pragma unroll
+    for (unsigned w = 0; w < SMALL_THREADS / 32; ++w) {
+        base += w < warp ? s_warp[w] : 0u;
+        block_max = max(block_max, s_max[w]);
+    }
+#pragma unroll
+    for (int q = 0; q < PER / 4; ++q) {
+        const uint4 u = make_uint4(base + v[4 * q], base + v[4 * q + 1], base + v[4 * q + 2], base + v[4 * q + 3]);
+        reinterpret_cast<uint4*>(s_off)[tid * (PER / 4) + q] = u;
+        const uint32_t c0 = tid * PER + 4 * q;
+        if (c0 < C) reinterpret_cast<uint4*>(offsets)[c0 / 4] = u;
+    }
+    // the control block: every word cleared but the error and M_C
+    constexpr uint32_t ERROR_WORD = offsetof(Ctrl, error) / 4, MAX_WORD = offsetof(Ctrl, max_per_cell) / 4;
+    if (tid < sizeof(Ctrl) / 4)
+        reinterpret_cast<uint32_t*>(ctrl)[tid] =
+            tid == ERROR_WORD ? (ok ? 0u : (uint32_t)ERR_OUT_OF_BOX) : (tid == MAX_WORD ? block_max : 0u);
+    if (tid == 0) {
+        pbase[0] = 0u;
+        pbase[1] = n;
+    }
+    for (uint32_t k = tid; k < C; k += SMALL_THREADS) xbins[k] = make_uint2(0u, 0u);
+    __syncthreads();
+    if (tid == 0) offsets[C] = n;  // (after the padded store of the last group)
+    if (!ok) return;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        const uint32_t i = tid + j * SMALL_THREADS;
+        if (i >= n) continue;
+        const float px = x[i];
+        const uint2 t = sub_bin_thermometer(px, c[j], d.g);
+        const uint32_t slot = s_off[c[j]] + r[j];
+        if (PI_BOUNDS(ctrl, slot, n, CS_SCATTER_REC)) store_rec(rec + slot, px, i, t.x, t.y, y[i], z[i], c[j]);
+    }
+}
+
 // Resident CTAs per SM of a binning kernel (256 threads, no dynamic shared
 // memory) on the current device, queried once per device and kernel.
 template <class F>
@@ -585,6 +695,14 @@ cudaError_t launch_stabilise(const Rec* rec, uint32_t n, const Systems& sy, cons
 {
     return launch_dependent(k_stabilise, dim3(grid_for(n, 256, num_sms, resident_per_sm(k_stabilise, 2))), dim3(256),
                             0, s, rec, n, sy, offsets, perm, sx, sy_out, sz, P, xbins, ctrl);
+}
+
+cudaError_t launch_bin_small(const float* x, const float* y, const float* z, uint32_t n, const Systems& sy, uint32_t C,
+                             uint32_t* pbase, uint32_t* counts, uint32_t* offsets, uint2* xbins, Rec* rec, Ctrl* ctrl,
+                             cudaStream_t s)
+{
+    return launch_dependent(k_bin_small, dim3(1), dim3(SMALL_THREADS), 0, s, x, y, z, n, sy, C, pbase, counts,
+                            offsets, xbins, rec, ctrl);
 }
 
 namespace {

@@ -432,6 +432,14 @@ cudaError_t launch_stabilise(const Rec* rec, uint32_t n,
                              float* sy_out, float* sz, float4* P, uint2* xbins, Ctrl* ctrl,
                              int num_sms, cudaStream_t s);
 
+// a1 - a4's first half of one system of at most SMALL_MAX particles in at
+// most SMALL_MAX cells in one launch (k_bin_small).
+constexpr int SMALL_THREADS = 1024;
+constexpr uint32_t SMALL_MAX = 4096;
+cudaError_t launch_bin_small(const float* x, const float* y, const float* z, uint32_t n, const Systems& sy, uint32_t C,
+                             uint32_t* pbase, uint32_t* counts, uint32_t* offsets, uint2* xbins, Rec* rec, Ctrl* ctrl,
+                             cudaStream_t s);
+
 // FP64 total of v over the particles of each system (out[S], device), in a
 // fixed order: `parts` partial sums per system in `partial` [S * parts].
 constexpr int TOTAL_PARTS = 32;
