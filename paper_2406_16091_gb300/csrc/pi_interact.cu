@@ -1957,35 +1957,13 @@ __host__ __device__ constexpr int direct4_min_blocks()
     return (std::is_same<Acc, PlainAcc>::value && (KERNEL == KERNEL_GAUSSIAN || KERNEL == KERNEL_LOWFLOP)) ? 5 : 1;
 }
 
-// Four targets per thread: P slots 4p .. 4p + 3.  Each source read feeds
-// four targets (two packed pairs), so the L1 reads per evaluation halve
-// while the union of four windows adds evaluations -- the better trade at
-// high occupancy (32 per cell), the worse at low.  Four slots lie in one
-// X-row of one system unless some are sentinels (every row ends in
-// ROW_PADS of them), which repeat a real target and store nothing.  Grids
-// with dense cells take the slot pairs' dense path.
-template <class Acc, int KERNEL, bool COUNT = false>
-__global__ void __launch_bounds__(DIRECT_THREADS, (direct4_min_blocks<Acc, KERNEL>()))
-    k_interact_direct4(InteractArgs a)
+// P slots k0 .. k0 + 3 below kend.  Four slots lie in one X-row of one system
+// unless some are sentinels (every row ends in ROW_PADS of them), which
+// repeat a real target and store nothing.
+template <bool DENSE, class Acc, int KERNEL, bool COUNT = false>
+__device__ __forceinline__ void direct_slot_quad(const InteractArgs& a, uint32_t (*win)[DIRECT_THREADS], unsigned col,
+                                                 uint32_t k0, uint32_t kend)
 {
-    __shared__ uint32_t win[20][DIRECT_THREADS];  // 9 windows (lo, hi) + one spare read after the last
-    pdl_wait();  // the binning (or the previous interaction) has completed
-    // keep the work counters of the tiled launches in step (see k_interact_tiled)
-    if (blockIdx.x == 0 && threadIdx.x == 0) a.ctrl->work[(a.seq + 1u) & 1u] = 0u;
-    // both control words in flight together, per thread (a per-CTA read
-    // and barrier, cta_ctrl_words, measured 1 % slower here: the
-    // evaluation hides these reads)
-    const uint32_t err = load_error(a.ctrl);
-    const uint32_t mpc = *((volatile const uint32_t*)&a.ctrl->max_per_cell);
-    if (err) return;
-    uint32_t k0, kend;
-    group_slots(a, 4u, k0, kend);
-    if (k0 >= kend) return;
-    if (mpc > DENSE_CELL) {
-        direct_slot_pair_dense<Acc, KERNEL, COUNT>(a, win, threadIdx.x, k0, kend);
-        direct_slot_pair_dense<Acc, KERNEL, COUNT>(a, win, threadIdx.x, k0 + 2u, kend);
-        return;
-    }
     constexpr uint32_t NONE = 0xffffffffu;
     float4 t[4];
     bool v[4];
@@ -2011,12 +1989,50 @@ __global__ void __launch_bounds__(DIRECT_THREADS, (direct4_min_blocks<Acc, KERNE
     const KParams kp = kparams(a, sid);
     Sums<Acc, KERNEL> r[4];
     const uint32_t slots =
-        direct_group<DIRECT_THREADS, 4, false, Acc, KERNEL, COUNT>(a, d, win, threadIdx.x, t, cx, cy, cz, kp, r);
+        direct_group<DIRECT_THREADS, 4, DENSE, Acc, KERNEL, COUNT>(a, d, win, col, t, cx, cy, cz, kp, r);
     add_evals<COUNT>(a, (unsigned long long)slots * ((v[0] ? 1u : 0u) + (v[1] ? 1u : 0u) + (v[2] ? 1u : 0u) +
                                               (v[3] ? 1u : 0u)));
 #pragma unroll
     for (int k = 0; k < 4; ++k)
         if (v[k]) store_out(a, __float_as_uint(t[k].w), r[k]);
+}
+
+// The four slots with exact window bounds in dense cells, out of line so that
+// the common path keeps its code and registers.  (Measured in us against the
+// two-target dense path twice per thread, clustered layouts: 600,000 at 16
+// per cell 1517 / 1121, 600,000 at 8 852 / 704, 400,000 at 10 679 / 529.)
+template <class Acc, int KERNEL, bool COUNT = false>
+__device__ __noinline__ void direct_slot_quad_dense(const InteractArgs& a, uint32_t (*win)[DIRECT_THREADS],
+                                                    unsigned col, uint32_t k0, uint32_t kend)
+{
+    direct_slot_quad<true, Acc, KERNEL, COUNT>(a, win, col, k0, kend);
+}
+
+// Four targets per thread: P slots 4p .. 4p + 3.  Each source read feeds
+// four targets (two packed pairs), so the L1 reads per evaluation halve
+// while the union of four windows adds evaluations -- the better trade at
+// high occupancy (32 per cell), the worse at low.
+template <class Acc, int KERNEL, bool COUNT = false>
+__global__ void __launch_bounds__(DIRECT_THREADS, (direct4_min_blocks<Acc, KERNEL>()))
+    k_interact_direct4(InteractArgs a)
+{
+    __shared__ uint32_t win[20][DIRECT_THREADS];  // 9 windows (lo, hi) + one spare read after the last
+    pdl_wait();  // the binning (or the previous interaction) has completed
+    // keep the work counters of the tiled launches in step (see k_interact_tiled)
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.ctrl->work[(a.seq + 1u) & 1u] = 0u;
+    // both control words in flight together, per thread (a per-CTA read
+    // and barrier, cta_ctrl_words, measured 1 % slower here: the
+    // evaluation hides these reads)
+    const uint32_t err = load_error(a.ctrl);
+    const uint32_t mpc = *((volatile const uint32_t*)&a.ctrl->max_per_cell);
+    if (err) return;
+    uint32_t k0, kend;
+    group_slots(a, 4u, k0, kend);
+    if (k0 >= kend) return;
+    if (mpc > DENSE_CELL)
+        direct_slot_quad_dense<Acc, KERNEL, COUNT>(a, win, threadIdx.x, k0, kend);
+    else
+        direct_slot_quad<false, Acc, KERNEL, COUNT>(a, win, threadIdx.x, k0, kend);
 }
 
 // The forms with a counting copy of the direct kernels (PI_OPT_COUNT_EVALS).
