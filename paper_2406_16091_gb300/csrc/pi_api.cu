@@ -518,6 +518,17 @@ pi_status pi_binned(const pi_ctx* ctx, const uint32_t** counts, const uint32_t**
     return PI_OK;
 }
 
+// Whether ptr is memory that was allocated on the context's device.
+static bool own_memory(const pi_ctx* ctx, const void* ptr)
+{
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, ptr) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeDevice && at.device == ctx->device;
+}
+
 pi_status pi_copy_binned(const pi_ctx* ctx, uint32_t* counts, uint32_t* offsets, uint32_t* perm,
                          float* sx, float* sy, float* sz, pi_stream stream)
 {
@@ -530,20 +541,27 @@ pi_status pi_copy_binned(const pi_ctx* ctx, uint32_t* counts, uint32_t* offsets,
     const void* src[6] = {ctx->counts, ctx->offsets, ctx->perm, ctx->sx, ctx->sy, ctx->sz};
     void* dst[6] = {counts, offsets, perm, sx, sy, sz};
     const size_t words[6] = {C, C + 1, n, n, n, n};
-    // one dependent launch for all the arrays; a destination that is not
-    // word-aligned goes by a memory copy (step with one array copied after
-    // it, by a memory copy / by this launch: 26.9 / 25.7 us at 1,531
-    // particles, 35.1 / 33.9 at 32,768, 441 / 437 for 64 systems)
+    // One dependent launch for all the arrays (step with one array copied
+    // after it, by a memory copy / by this launch: 26.9 / 25.7 us at 1,531
+    // particles, 35.1 / 33.9 at 32,768, 441 / 437 for 64 systems).  It writes
+    // by plain stores and in no order, so memory copies, one after the other,
+    // stay for destinations that are not word-aligned, not memory of this
+    // device (host or another device's memory), or that overlap.
     pi::CopyArgs c{};
+    bool plain = true;
     for (int k = 0; k < 6; ++k) {
         if (!dst[k] || words[k] == 0) continue;
-        if ((uintptr_t)dst[k] % 4 != 0) {
-            PI_TRY(cudaMemcpyAsync(dst[k], src[k], words[k] * 4, cudaMemcpyDeviceToDevice, s));
-            continue;
-        }
+        plain = plain && (uintptr_t)dst[k] % 4 == 0 && own_memory(ctx, dst[k]);
+        for (int j = 0; j < c.count; ++j)
+            plain = plain && ((uint32_t*)dst[k] + words[k] <= c.dst[j] || c.dst[j] + c.words[j] <= (uint32_t*)dst[k]);
         c.src[c.count] = (const uint32_t*)src[k];
         c.dst[c.count] = (uint32_t*)dst[k];
         c.words[c.count++] = words[k];
+    }
+    if (!plain) {
+        for (int k = 0; k < c.count; ++k)
+            PI_TRY(cudaMemcpyAsync(c.dst[k], c.src[k], c.words[k] * 4, cudaMemcpyDeviceToDevice, s));
+        return PI_OK;
     }
     if (c.count > 0) {
         PI_TRY(pi::launch_copy_words(c, s));

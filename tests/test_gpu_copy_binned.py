@@ -38,3 +38,29 @@ def test_copies_every_subset_and_alignment(n, cells, shift, names):
             assert np.all(a[:shift] == -7) and np.all(a[shift + m:] == -7), k
     finally:
         B.pi_destroy(ctx)
+
+
+def test_memory_copies_for_host_memory_and_shared_destinations():
+    # Destinations that the launch must not write: page-locked host memory,
+    # and one buffer named twice (the array copied last stands).
+    torch = pytest.importorskip("torch")
+    dev = torch.device("cuda", 0)
+    n, rc = 4099, W.rc_for_cells(8)
+    x, y, z = W.uniform(n, 17)
+    b = oracle.bin_particles(x, y, z, (0, 0, 0), (1, 1, 1), rc)
+    s = torch.cuda.current_stream()
+    ctx = B.pi_create((0, 0, 0), (1, 1, 1), rc, n)
+    try:
+        t = [torch.from_numpy(a).to(dev) for a in (x, y, z)]
+        B.pi_bin(ctx, *t, n, s)
+        host = torch.zeros(n, dtype=torch.int32).pin_memory()
+        both = torch.zeros(n, dtype=torch.int32, device=dev)
+        launched = B.pi_launch_count(ctx)
+        B.pi_copy_binned(ctx, perm=host, stream=s)
+        B.pi_copy_binned(ctx, perm=both, sz=both, stream=s)
+        B.pi_sync_status(ctx, s)
+        assert B.pi_launch_count(ctx) == launched
+        assert np.array_equal(host.numpy().view(np.uint32), b.perm)
+        assert np.array_equal(both.cpu().numpy().view(np.uint32), b.sz.view(np.uint32))
+    finally:
+        B.pi_destroy(ctx)
