@@ -70,6 +70,10 @@ struct pi_ctx {
     std::vector<uint32_t> pbase_h;  // [S+1] particle bases of the last pi_bin
     std::vector<float> kscale_h;    // [2S] per-system kernel scales last written to d_kscale
     int binned;                     // a pi_bin has been enqueued since the last failure
+    // the stream and capture (0: none) of the last pi_bin, whose records
+    // pi_interact on the same stream may write over (see record_stream)
+    unsigned long long bin_stream, bin_capture;
+    bool bin_stream_known;
     uint32_t epoch;                 // scan launch epoch
     mutable uint64_t launches;      // kernels launched
     uint32_t tiled_seq;             // launches of the tiled interaction kernel
@@ -518,6 +522,30 @@ pi_status pi_binned(const pi_ctx* ctx, const uint32_t** counts, const uint32_t**
     return PI_OK;
 }
 
+// Input-order outputs go through the binning's records (launch_unpermute)
+// from this many particles on (see records_pay).
+constexpr int64_t UNPERMUTE_MIN = 1000000;
+
+// The identity of a stream and of the capture it is in (0: none); false if
+// either is not to be had.  The records belong to the stream, and capture, of
+// the last pi_bin: interactions there follow one another, so one pair of
+// kernels is done with the records before the next writes them.  One on
+// another stream, or captured alone, may overlap and writes to its arrays.
+static bool record_stream(cudaStream_t s, unsigned long long* stream, unsigned long long* capture)
+{
+    if (s == cudaStreamPerThread) return false;  // one handle, a stream per host thread
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    *capture = 0;
+    cudaError_t e = cudaStreamGetCaptureInfo(s, &cap, capture);
+    if (cap == cudaStreamCaptureStatusActive)
+        *stream = (unsigned long long)(uintptr_t)s;  // cudaStreamGetId would end the capture
+    else
+        e = e == cudaSuccess ? cudaStreamGetId(s, stream) : e;
+    if (e != cudaSuccess) (void)cudaGetLastError();
+    if (cap == cudaStreamCaptureStatusNone) *capture = 0;
+    return e == cudaSuccess && cap != cudaStreamCaptureStatusInvalidated;
+}
+
 // Whether ptr is memory that was allocated on the context's device.
 static bool own_memory(const pi_ctx* ctx, const void* ptr)
 {
@@ -646,6 +674,8 @@ pi_status pi_batch_bin(pi_ctx* ctx, const float* x, const float* y, const float*
     if (ds.err != cudaSuccess) return cuda_fail(ds.err, "pi_bin: set device");
     cudaStream_t s = (cudaStream_t)stream;
     ctx->binned = 0;
+    ctx->bin_stream_known =
+        total >= UNPERMUTE_MIN && record_stream(s, &ctx->bin_stream, &ctx->bin_capture);
     ctx->tiled_seq = 0;  // k_zero clears both row-counter slots
     ctx->epoch = (ctx->epoch % 0x3ffffffeu) + 1u;  // 30-bit, never 0
     ctx->pbase_h[0] = 0;
@@ -857,6 +887,34 @@ bool one_target_form(const pi_ctx* ctx, int kernel)
     return ctx->precision == PI_PREC_KAHAN && ctx->n < 6 * ctx->C;
 }
 
+// Whether input-order outputs go through records and k_unpermute instead of
+// straight to the arrays: in the two- and four-target direct kernels with
+// plain Gaussian or low-FLOP sums (recorded_form).  The extra pass costs about
+// 5 us per million particles.  Against it stand the scattered words, which a
+// long evaluation hides as long as the L2 holds the arrays.  Medians of a
+// step in us, straight / records (particles, mean per cell):
+//   - two targets per thread: 600,000 at 1 75.6 / 77.7 (an earlier k_unpermute),
+//     1 M at 1 121.8 / 114.4 and at 4 140 / 136, 1.5 M at 2 182 / 169, 2 M at
+//     1 251 / 230 and at 6 319 / 303, 16.8 M at 1 3294 / 2018, clustered 2 M
+//     at 1 516 / 514 and at 2 810 / 797;
+//   - four targets, whose evaluation is longer, from n = 65536 q^2 at q per
+//     cell: 2 M at 8 324 / 335, 3 M at 8 454 / 470, 4.2 M at 8 678 / 652, 8.4 M
+//     at 8 1540 / 1334, 4.2 M at 12 756 / 786, 8.4 M at 12 1593 / 1576, 16.8 M
+//     at 16 3697 / 3710 and at 32 5704 / 5909.
+bool records_pay(const pi_ctx* ctx, const pi::InteractArgs& a)
+{
+    if (ctx->algo == PI_ALGO_PPNL || ctx->precision == PI_PREC_KAHAN || ctx->count_evals || a.one_target) return false;
+    if (a.kernel != pi::KERNEL_GAUSSIAN && a.kernel != pi::KERNEL_LOWFLOP) return false;
+    // every target of the launch must be written: direct shapes, no system left out
+    if (ctx->sys_tile.empty() ? (ctx->tile >= 0 && ctx->tile < pi::DEFAULT_TILE)
+                              : std::find(ctx->sys_tile.begin(), ctx->sys_tile.end(), 0) != ctx->sys_tile.end())
+        return false;
+    const double n = (double)ctx->n, C = (double)ctx->C;
+    if (ctx->n < UNPERMUTE_MIN) return false;
+    if (n < 8 * C) return n < 4 * C || n >= 1.5 * (double)UNPERMUTE_MIN;
+    return C * C >= 65536.0 * n;
+}
+
 // Occupancy regimes of the per-system autotuning: mean particles per cell
 // below 4, below 8, and from 8 on (the shapes' crossover is near 8).
 int occupancy_regime(const pi_ctx* ctx, int s)
@@ -945,6 +1003,10 @@ pi_status pi_batch_interact(pi_ctx* ctx, const float* h, float* S, float* Vx, fl
     a.seq = ctx->tiled_seq;
     a.count_evals = ctx->count_evals;
     a.one_target = one_target_form(ctx, a.kernel);
+    unsigned long long stream_id = 0, capture_id = 0;
+    if (a.original_order && records_pay(ctx, a) && ctx->bin_stream_known &&
+        record_stream(st, &stream_id, &capture_id) && stream_id == ctx->bin_stream && capture_id == ctx->bin_capture)
+        a.orec = reinterpret_cast<uint4*>(ctx->rec);
     int launched = 0;
     cudaError_t e;
     const bool kahan = ctx->precision == PI_PREC_KAHAN;
@@ -952,9 +1014,10 @@ pi_status pi_batch_interact(pi_ctx* ctx, const float* h, float* S, float* Vx, fl
         e = pi::launch_interact_ppnl(a, kahan, ctx->num_sms, st, &launched);
     } else if (!ctx->sys_tile.empty()) {
         const pi_status ps = launch_plan(ctx, a, kahan, st, &launched);
+        e = ps == PI_OK && a.orec ? pi::launch_unpermute(a, st, &launched) : cudaSuccess;
         ctx->launches += (uint64_t)launched;
         ctx->tiled_seq += 1;
-        return ps;
+        return e != cudaSuccess ? cuda_fail(e, "pi_interact: launch") : ps;
     } else {
         // PI_TILE_AUTO: four targets per thread for the plain Gaussian and
         // low-FLOP sums from 8 particles per cell on average (measured
@@ -979,6 +1042,7 @@ pi_status pi_batch_interact(pi_ctx* ctx, const float* h, float* S, float* Vx, fl
                                       &launched);
         ctx->tiled_seq += 1;
     }
+    if (e == cudaSuccess && a.orec) e = pi::launch_unpermute(a, st, &launched);
     ctx->launches += (uint64_t)launched;
     if (e != cudaSuccess) return cuda_fail(e, "pi_interact: launch");
     return PI_OK;

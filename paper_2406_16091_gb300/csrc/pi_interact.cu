@@ -245,17 +245,31 @@ struct Sums {
     }
 };
 
-template <class Acc, int KERNEL>
+// Forms of the direct kernels: outputs to the arrays; the same, counting
+// evaluations (PI_OPT_COUNT_EVALS); outputs as records by input index (see
+// k_unpermute).  A form per copy, since a test of it in the one kernel cost
+// the others 2 to 3 % (scale 233 / 238, clustered 1274 / 1313 us).
+enum : int { FORM_PLAIN = 0, FORM_COUNT = 1, FORM_RECORD = 2 };
+
+template <int FORM = FORM_PLAIN, class Acc, int KERNEL>
 __device__ __forceinline__ void store_out(const InteractArgs& a, uint32_t slot, const Sums<Acc, KERNEL>& r)
 {
     if (!PI_BOUNDS(a.ctrl, slot, a.n, CS_DIRECT_TARGET)) return;
-    const uint32_t o = a.original_order ? a.perm[slot] : slot;
+    const uint32_t o = FORM == FORM_RECORD || a.original_order ? a.perm[slot] : slot;
     if (!PI_BOUNDS(a.ctrl, o, a.n, CS_DIRECT_TARGET)) return;
-    a.S[o] = r.s.value();
-    a.Vx[o] = r.vx.value();
-    a.Vy[o] = r.vy.value();
-    a.Vz[o] = r.vz.value();
-    if (a.nbr) a.nbr[o] = r.n;
+    if constexpr (FORM == FORM_RECORD) {
+        // one whole sector instead of five words in five
+        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %6, %6};" ::"l"(a.orec + 2 * (size_t)o),
+                     "r"(__float_as_uint(r.s.value())), "r"(__float_as_uint(r.vx.value())),
+                     "r"(__float_as_uint(r.vy.value())), "r"(__float_as_uint(r.vz.value())), "r"(r.n), "r"(0u)
+                     : "memory");
+    } else {
+        a.S[o] = r.s.value();
+        a.Vx[o] = r.vx.value();
+        a.Vy[o] = r.vy.value();
+        a.Vz[o] = r.vz.value();
+        if (a.nbr) a.nbr[o] = r.n;
+    }
 }
 
 // ---- Alg. 1: Par-Part-NoLoop ------------------------------------------------
@@ -1585,8 +1599,8 @@ __device__ __forceinline__ void group_windows(const InteractArgs& a, const SysDe
 // four targets one before a window's start -- add exact zeros, so each
 // target's sums are those of the sequential loop over its own windows.
 // Returns the source slots each target is evaluated against (the windows
-// rounded up to whole four-source trips) in the counting copy (COUNT), else 0.
-template <int WT, int G, bool DENSE, class Acc, int KERNEL, bool COUNT = false>
+// rounded up to whole four-source trips) in the counting copy, else 0.
+template <int WT, int G, bool DENSE, class Acc, int KERNEL, int FORM = FORM_PLAIN>
 __device__ __forceinline__ uint32_t direct_group(const InteractArgs& a, const SysDesc& d, uint32_t (*win)[WT],
                                                  unsigned col, const float4 (&t)[G], const int (&cx)[G], int cy,
                                                  int cz, const KParams& kp, Sums<Acc, KERNEL> (&r)[G])
@@ -1616,7 +1630,7 @@ __device__ __forceinline__ uint32_t direct_group(const InteractArgs& a, const Sy
                 const uint32_t lo = WIDE ? ulo[rr] & ~1u : ulo[rr];
                 win[2 * nw][col] = lo;
                 win[2 * nw + 1][col] = uhi[rr];
-                if constexpr (COUNT) slots += (uhi[rr] - lo + 3u) & ~3u;
+                if constexpr (FORM == FORM_COUNT) slots += (uhi[rr] - lo + 3u) & ~3u;
                 ++nw;
             }
     }
@@ -1698,10 +1712,10 @@ __device__ __forceinline__ uint32_t direct_group(const InteractArgs& a, const Sy
 
 // Adds a thread's counted evaluations to the control block (the counting
 // copy of the direct kernels, PI_OPT_COUNT_EVALS: one atomic per thread).
-template <bool COUNT>
+template <int FORM>
 __device__ __forceinline__ void add_evals(const InteractArgs& a, unsigned long long ev)
 {
-    if constexpr (COUNT) {
+    if constexpr (FORM == FORM_COUNT) {
         if (ev) atomicAdd(&a.ctrl->evals, ev);
     }
 }
@@ -1726,7 +1740,7 @@ __device__ __forceinline__ void group_slots(const InteractArgs& a, uint32_t per,
 
 // Slots ka and ka + 1 of P below kend (either may be a sentinel or past
 // the end).
-template <int WT, bool DENSE, class Acc, int KERNEL, bool COUNT = false>
+template <int WT, bool DENSE, class Acc, int KERNEL, int FORM = FORM_PLAIN>
 __device__ __forceinline__ void direct_slot_pair(const InteractArgs& a, uint32_t (*win)[WT], unsigned col,
                                                  uint32_t ka, uint32_t kend)
 {
@@ -1759,10 +1773,10 @@ __device__ __forceinline__ void direct_slot_pair(const InteractArgs& a, uint32_t
         const float4 t[2] = {ta, together ? t1 : ta};
         const int cx[2] = {cxa, together ? cxb : cxa};
         Sums<Acc, KERNEL> r[2];
-        const uint32_t slots = direct_group<WT, 2, DENSE, Acc, KERNEL, COUNT>(a, d, win, col, t, cx, cy, cz, kp, r);
-        add_evals<COUNT>(a, (unsigned long long)slots * (together ? 2u : 1u));
-        store_out(a, __float_as_uint(ta.w), r[0]);
-        if (together) store_out(a, __float_as_uint(t1.w), r[1]);
+        const uint32_t slots = direct_group<WT, 2, DENSE, Acc, KERNEL, FORM>(a, d, win, col, t, cx, cy, cz, kp, r);
+        add_evals<FORM>(a, (unsigned long long)slots * (together ? 2u : 1u));
+        store_out<FORM>(a, __float_as_uint(ta.w), r[0]);
+        if (together) store_out<FORM>(a, __float_as_uint(t1.w), r[1]);
     }
     if (has_b && !together) {
         const SysDesc& d1 = a.sy.sys[sid1];
@@ -1774,18 +1788,18 @@ __device__ __forceinline__ void direct_slot_pair(const InteractArgs& a, uint32_t
         const float4 t[2] = {t1, t1};
         const int cx[2] = {cx1, cx1};
         Sums<Acc, KERNEL> r[2];
-        add_evals<COUNT>(a, direct_group<WT, 2, DENSE, Acc, KERNEL, COUNT>(a, d1, win, col, t, cx, cy1, cz1, kp1, r));
-        store_out(a, __float_as_uint(t1.w), r[0]);
+        add_evals<FORM>(a, direct_group<WT, 2, DENSE, Acc, KERNEL, FORM>(a, d1, win, col, t, cx, cy1, cz1, kp1, r));
+        store_out<FORM>(a, __float_as_uint(t1.w), r[0]);
     }
 }
 
 // The slot pair with exact window bounds in dense cells, out of line so that
 // the common path keeps its code and registers.
-template <class Acc, int KERNEL, bool COUNT = false>
+template <class Acc, int KERNEL, int FORM = FORM_PLAIN>
 __device__ __noinline__ void direct_slot_pair_dense(const InteractArgs& a, uint32_t (*win)[DIRECT_THREADS],
                                                     unsigned col, uint32_t ka, uint32_t kend)
 {
-    direct_slot_pair<DIRECT_THREADS, true, Acc, KERNEL, COUNT>(a, win, col, ka, kend);
+    direct_slot_pair<DIRECT_THREADS, true, Acc, KERNEL, FORM>(a, win, col, ka, kend);
 }
 
 // Resident CTAs per SM the direct kernel's registers are capped for.  The
@@ -1800,9 +1814,9 @@ __host__ __device__ constexpr int direct_min_blocks()
     return (std::is_same<Acc, PlainAcc>::value && (KERNEL == KERNEL_GAUSSIAN || KERNEL == KERNEL_LOWFLOP)) ? 8 : 6;
 }
 
-// Targets of P slots 2p and 2p + 1 per thread.  COUNT: the copy that also
-// counts its evaluations (PI_OPT_COUNT_EVALS).
-template <class Acc, int KERNEL, bool COUNT = false>
+// Targets of P slots 2p and 2p + 1 per thread.  FORM: the plain copy, the one
+// that counts its evaluations, or the one that writes records.
+template <class Acc, int KERNEL, int FORM = FORM_PLAIN>
 __global__ void __launch_bounds__(DIRECT_THREADS, (direct_min_blocks<Acc, KERNEL>()))
     k_interact_direct(InteractArgs a)
 {
@@ -1821,9 +1835,9 @@ __global__ void __launch_bounds__(DIRECT_THREADS, (direct_min_blocks<Acc, KERNEL
     uint32_t k0, kend;
     group_slots(a, 2u, k0, kend);
     if (mpc > DENSE_CELL)
-        direct_slot_pair_dense<Acc, KERNEL, COUNT>(a, win, threadIdx.x, k0, kend);
+        direct_slot_pair_dense<Acc, KERNEL, FORM>(a, win, threadIdx.x, k0, kend);
     else
-        direct_slot_pair<DIRECT_THREADS, false, Acc, KERNEL, COUNT>(a, win, threadIdx.x, k0, kend);
+        direct_slot_pair<DIRECT_THREADS, false, Acc, KERNEL, FORM>(a, win, threadIdx.x, k0, kend);
 }
 
 // ---- one target per thread ----
@@ -1960,7 +1974,7 @@ __host__ __device__ constexpr int direct4_min_blocks()
 // P slots k0 .. k0 + 3 below kend.  Four slots lie in one X-row of one system
 // unless some are sentinels (every row ends in ROW_PADS of them), which
 // repeat a real target and store nothing.
-template <bool DENSE, class Acc, int KERNEL, bool COUNT = false>
+template <bool DENSE, class Acc, int KERNEL, int FORM = FORM_PLAIN>
 __device__ __forceinline__ void direct_slot_quad(const InteractArgs& a, uint32_t (*win)[DIRECT_THREADS], unsigned col,
                                                  uint32_t k0, uint32_t kend)
 {
@@ -1989,30 +2003,30 @@ __device__ __forceinline__ void direct_slot_quad(const InteractArgs& a, uint32_t
     const KParams kp = kparams(a, sid);
     Sums<Acc, KERNEL> r[4];
     const uint32_t slots =
-        direct_group<DIRECT_THREADS, 4, DENSE, Acc, KERNEL, COUNT>(a, d, win, col, t, cx, cy, cz, kp, r);
-    add_evals<COUNT>(a, (unsigned long long)slots * ((v[0] ? 1u : 0u) + (v[1] ? 1u : 0u) + (v[2] ? 1u : 0u) +
+        direct_group<DIRECT_THREADS, 4, DENSE, Acc, KERNEL, FORM>(a, d, win, col, t, cx, cy, cz, kp, r);
+    add_evals<FORM>(a, (unsigned long long)slots * ((v[0] ? 1u : 0u) + (v[1] ? 1u : 0u) + (v[2] ? 1u : 0u) +
                                               (v[3] ? 1u : 0u)));
 #pragma unroll
     for (int k = 0; k < 4; ++k)
-        if (v[k]) store_out(a, __float_as_uint(t[k].w), r[k]);
+        if (v[k]) store_out<FORM>(a, __float_as_uint(t[k].w), r[k]);
 }
 
 // The four slots with exact window bounds in dense cells, out of line so that
 // the common path keeps its code and registers.  (Measured in us against the
 // two-target dense path twice per thread, clustered layouts: 600,000 at 16
 // per cell 1517 / 1121, 600,000 at 8 852 / 704, 400,000 at 10 679 / 529.)
-template <class Acc, int KERNEL, bool COUNT = false>
+template <class Acc, int KERNEL, int FORM = FORM_PLAIN>
 __device__ __noinline__ void direct_slot_quad_dense(const InteractArgs& a, uint32_t (*win)[DIRECT_THREADS],
                                                     unsigned col, uint32_t k0, uint32_t kend)
 {
-    direct_slot_quad<true, Acc, KERNEL, COUNT>(a, win, col, k0, kend);
+    direct_slot_quad<true, Acc, KERNEL, FORM>(a, win, col, k0, kend);
 }
 
 // Four targets per thread: P slots 4p .. 4p + 3.  Each source read feeds
 // four targets (two packed pairs), so the L1 reads per evaluation halve
 // while the union of four windows adds evaluations -- the better trade at
 // high occupancy (32 per cell), the worse at low.
-template <class Acc, int KERNEL, bool COUNT = false>
+template <class Acc, int KERNEL, int FORM = FORM_PLAIN>
 __global__ void __launch_bounds__(DIRECT_THREADS, (direct4_min_blocks<Acc, KERNEL>()))
     k_interact_direct4(InteractArgs a)
 {
@@ -2030,9 +2044,9 @@ __global__ void __launch_bounds__(DIRECT_THREADS, (direct4_min_blocks<Acc, KERNE
     group_slots(a, 4u, k0, kend);
     if (k0 >= kend) return;
     if (mpc > DENSE_CELL)
-        direct_slot_quad_dense<Acc, KERNEL, COUNT>(a, win, threadIdx.x, k0, kend);
+        direct_slot_quad_dense<Acc, KERNEL, FORM>(a, win, threadIdx.x, k0, kend);
     else
-        direct_slot_quad<false, Acc, KERNEL, COUNT>(a, win, threadIdx.x, k0, kend);
+        direct_slot_quad<false, Acc, KERNEL, FORM>(a, win, threadIdx.x, k0, kend);
 }
 
 // The forms with a counting copy of the direct kernels (PI_OPT_COUNT_EVALS).
@@ -2040,6 +2054,14 @@ template <class Acc, int KERNEL>
 constexpr bool counted_form()
 {
     return std::is_same<Acc, PlainAcc>::value && (KERNEL == KERNEL_GAUSSIAN || KERNEL == KERNEL_GAUSSIAN_FINE);
+}
+
+// The forms with a copy that writes records (the host sets a.orec for no
+// other, see records_pay).
+template <class Acc, int KERNEL>
+constexpr bool recorded_form()
+{
+    return std::is_same<Acc, PlainAcc>::value && (KERNEL == KERNEL_GAUSSIAN || KERNEL == KERNEL_LOWFLOP);
 }
 
 // Blocks of a direct launch: over all of P, or a.range_blocks for a launch
@@ -2059,7 +2081,14 @@ void launch_direct4_one(const InteractArgs& a, cudaStream_t s)
     // so the count, do not depend on the kernel K or the precision)
     if constexpr (counted_form<Acc, KERNEL>()) {
         if (a.count_evals) {
-            (void)launch_dependent(k_interact_direct4<Acc, KERNEL, true>, dim3(direct_grid(a, 4)),
+            (void)launch_dependent(k_interact_direct4<Acc, KERNEL, FORM_COUNT>, dim3(direct_grid(a, 4)),
+                                   dim3(DIRECT_THREADS), 0, s, a);
+            return;
+        }
+    }
+    if constexpr (recorded_form<Acc, KERNEL>()) {
+        if (a.orec) {
+            (void)launch_dependent(k_interact_direct4<Acc, KERNEL, FORM_RECORD>, dim3(direct_grid(a, 4)),
                                    dim3(DIRECT_THREADS), 0, s, a);
             return;
         }
@@ -2077,7 +2106,14 @@ void launch_direct_one(const InteractArgs& a, cudaStream_t s)
     // an error is left for cudaGetLastError
     if constexpr (counted_form<Acc, KERNEL>()) {
         if (a.count_evals) {
-            (void)launch_dependent(k_interact_direct<Acc, KERNEL, true>, dim3(direct_grid(a, 2)),
+            (void)launch_dependent(k_interact_direct<Acc, KERNEL, FORM_COUNT>, dim3(direct_grid(a, 2)),
+                                   dim3(DIRECT_THREADS), 0, s, a);
+            return;
+        }
+    }
+    if constexpr (recorded_form<Acc, KERNEL>()) {
+        if (a.orec) {
+            (void)launch_dependent(k_interact_direct<Acc, KERNEL, FORM_RECORD>, dim3(direct_grid(a, 2)),
                                    dim3(DIRECT_THREADS), 0, s, a);
             return;
         }
@@ -2181,6 +2217,49 @@ cudaError_t occupancy_of(int* per_sm)
 }
 
 }  // namespace
+
+// Input-order outputs of a large system.  Written straight to the arrays, each
+// target's five words fall into five sectors that hold nothing else of its
+// warp, and past the L2 each is a read and a write of 32 bytes in DRAM; the
+// interaction writes them as one record by input index instead (a whole
+// sector, so nothing is read), and this pass, bound by its 52 bytes per
+// particle, copies the records to the arrays in order.  Step of 2 M particles
+// at 1 per cell 251 -> 230 us, of 16.8 M 3294 -> 2018; one record of two
+// 16-byte loads per thread instead of two of one 256-bit load 238 and 2065.
+constexpr uint32_t UNPERMUTE_THREADS = 256, UNPERMUTE_PER_CTA = 2 * UNPERMUTE_THREADS;
+static __global__ void __launch_bounds__(UNPERMUTE_THREADS) k_unpermute(InteractArgs a)
+{
+    pdl_wait();
+    const uint32_t err = load_error(a.ctrl);
+    const uint32_t i0 = blockIdx.x * UNPERMUTE_PER_CTA + threadIdx.x;
+    uint32_t v[2][8];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const uint32_t i = min(i0 + k * UNPERMUTE_THREADS, a.n - 1u);
+        asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=r"(v[k][0]), "=r"(v[k][1]), "=r"(v[k][2]), "=r"(v[k][3]), "=r"(v[k][4]), "=r"(v[k][5]),
+                       "=r"(v[k][6]), "=r"(v[k][7])
+                     : "l"(a.orec + 2 * (size_t)i));
+    }
+    // after an error some records may be missing: the outputs stay as they are
+    if (err) return;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const uint32_t i = i0 + k * UNPERMUTE_THREADS;
+        if (i >= a.n) return;
+        a.S[i] = __uint_as_float(v[k][0]);
+        a.Vx[i] = __uint_as_float(v[k][1]);
+        a.Vy[i] = __uint_as_float(v[k][2]);
+        a.Vz[i] = __uint_as_float(v[k][3]);
+        if (a.nbr) a.nbr[i] = v[k][4];
+    }
+}
+
+cudaError_t launch_unpermute(const InteractArgs& a, cudaStream_t s, int* launches)
+{
+    *launches += 1;
+    return launch_dependent(k_unpermute, dim3((a.n - 1) / UNPERMUTE_PER_CTA + 1), dim3(UNPERMUTE_THREADS), 0, s, a);
+}
 
 cudaError_t launch_interact_ppnl(const InteractArgs& a, bool kahan, int num_sms, cudaStream_t s,
                                  int* launches)

@@ -502,6 +502,8 @@ struct InteractArgs {
     float* Vz;
     uint32_t* nbr;
     int original_order;
+    uint4* orec;            // original order through records (two uint4 per particle, by input index, see
+                            // launch_unpermute); null: straight to the arrays
     Ctrl* ctrl;
     uint64_t wait_limit_ns; // bound of every device-side wait
     uint32_t seq;           // launch number of the tiled kernel (row counter slot)
@@ -528,6 +530,8 @@ constexpr int DEFAULT_TILE = 5;         // PI_TILE_AUTO below 8 particles per ce
 constexpr int HIGH_OCCUPANCY_TILE = 6;  // PI_TILE_AUTO: plain Gaussian / low-FLOP sums from 8 per cell
 cudaError_t launch_interact_tiled(const InteractArgs& a, bool kahan, int num_sms, const int* per_sm,
                                   int tile, cudaStream_t s, int* launches);
+// The records of a.orec to the output arrays.
+cudaError_t launch_unpermute(const InteractArgs& a, cudaStream_t s, int* launches);
 // Resident CTAs per SM of each tile shape of the tiled kernel (per_sm[NUM_TILES]).
 cudaError_t tiled_occupancy(bool kahan, int* per_sm);
 
