@@ -889,7 +889,9 @@ bool one_target_form(const pi_ctx* ctx, int kernel)
 
 // Whether input-order outputs go through records and k_unpermute instead of
 // straight to the arrays: in the two- and four-target direct kernels with
-// plain Gaussian or low-FLOP sums (recorded_form).  The extra pass costs about
+// plain Gaussian, low-FLOP or Lennard-Jones sums (recorded_form; the
+// compensated sums hide the words throughout: 8.4 M at 8 2010 / 2036, 16.8 M
+// 4071 / 4137).  The extra pass costs about
 // 5 us per million particles.  Against it stand the scattered words, which a
 // long evaluation hides as long as the L2 holds the arrays.  Medians of a
 // step in us, straight / records (particles, mean per cell):
@@ -900,11 +902,13 @@ bool one_target_form(const pi_ctx* ctx, int kernel)
 //   - four targets, whose evaluation is longer, from n = 65536 q^2 at q per
 //     cell: 2 M at 8 324 / 335, 3 M at 8 454 / 470, 4.2 M at 8 678 / 652, 8.4 M
 //     at 8 1540 / 1334, 4.2 M at 12 756 / 786, 8.4 M at 12 1593 / 1576, 16.8 M
-//     at 16 3697 / 3710 and at 32 5704 / 5909.
+//     at 16 3697 / 3710 and at 32 5704 / 5909;
+//   - Lennard-Jones likewise: 1 M at 1 128 / 125, 2 M at 4 303 / 300, 8.4 M
+//     at 8 1616 / 1533, 16.8 M at 2 3713 / 2196 and at 16 4666 / 4605.
 bool records_pay(const pi_ctx* ctx, const pi::InteractArgs& a)
 {
     if (ctx->algo == PI_ALGO_PPNL || ctx->precision == PI_PREC_KAHAN || ctx->count_evals || a.one_target) return false;
-    if (a.kernel != pi::KERNEL_GAUSSIAN && a.kernel != pi::KERNEL_LOWFLOP) return false;
+    if (a.kernel != pi::KERNEL_GAUSSIAN && a.kernel != pi::KERNEL_LOWFLOP && a.kernel != pi::KERNEL_LJ) return false;
     // every target of the launch must be written: direct shapes, no system left out
     if (ctx->sys_tile.empty() ? (ctx->tile >= 0 && ctx->tile < pi::DEFAULT_TILE)
                               : std::find(ctx->sys_tile.begin(), ctx->sys_tile.end(), 0) != ctx->sys_tile.end())

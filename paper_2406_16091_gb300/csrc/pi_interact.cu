@@ -2061,7 +2061,8 @@ constexpr bool counted_form()
 template <class Acc, int KERNEL>
 constexpr bool recorded_form()
 {
-    return std::is_same<Acc, PlainAcc>::value && (KERNEL == KERNEL_GAUSSIAN || KERNEL == KERNEL_LOWFLOP);
+    return std::is_same<Acc, PlainAcc>::value &&
+           (KERNEL == KERNEL_GAUSSIAN || KERNEL == KERNEL_LOWFLOP || KERNEL == KERNEL_LJ);
 }
 
 // Blocks of a direct launch: over all of P, or a.range_blocks for a launch

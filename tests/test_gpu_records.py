@@ -49,7 +49,7 @@ def same(torch, a, b):
 @pytest.mark.parametrize("n,cells,records", [(EDGE - 1, 100, False), (EDGE, 100, True), (EDGE + 513, 70, True),
                                              (EDGE + 1, 60, False), (1500001, 60, True), (2097152, 64, False),
                                              (6000001, 90, True)])
-@pytest.mark.parametrize("kernel", [B.PI_KERNEL_GAUSSIAN, B.PI_KERNEL_LOWFLOP])
+@pytest.mark.parametrize("kernel", [B.PI_KERNEL_GAUSSIAN, B.PI_KERNEL_LOWFLOP, B.PI_KERNEL_LJ])
 @pytest.mark.parametrize("tile,shift,counts", [(-1, 0, True), (5, 1, True), (6, 3, False)])
 def test_records_equal_sorted_outputs(n, cells, records, kernel, tile, shift, counts):
     torch = pytest.importorskip("torch")
