@@ -45,7 +45,9 @@
 //                      the sorted order makes each one contiguous).
 //   k_interact_ws      the same chunks with a producer warp that stages them
 //                      for consumer warps (warp specialisation).
-// All of them sum each target's terms in the order of its own windows, so
+//   k_unpermute        after a direct kernel that left the outputs of a
+//                      large system as records by input index: to the arrays.
+// The others sum each target's terms in the order of its own windows, so
 // their outputs are bitwise equal.  Every one is a dependent launch: it waits
 // for the binning's last kernel (or the previous interaction) before reading
 // anything of the step.

@@ -17,7 +17,8 @@
 //   cell[n_max]     cell of each input particle            (binning scratch)
 //   rank[n_max]     provisional slot inside its cell        (binning scratch)
 //   rec[n_max]      32-byte Rec per particle in unstable slot order (binning
-//                   scratch): one full DRAM sector per random write
+//                   scratch): one full DRAM sector per random write; then
+//                   the input-order outputs of a large interaction
 //   perm[n_max]     stable   slot -> input index
 //   sx, sy, sz      positions in sorted order
 //   P[n_max]        float4 (x, y, z, stable slot): sorted order, and inside
