@@ -183,22 +183,32 @@ pi_status make_system(const pi_box& box, float r_c, SysDesc& d, int64_t& cells)
     return PI_OK;
 }
 
+// The power of two e that makes the Lennard-Jones scale e / sigma^2 a normal
+// FP32 number: 1 unless h^2 is below 2.9e-39 or above 8.5e37 (every h^2 that
+// FP32 holds lies between 2^-149 and 2^128).
+float lj_power(float h)
+{
+    const double t = 1.0 / ((double)h * (double)h);
+    return t > (double)FLT_MAX ? 0x1p-24f : (t < (double)FLT_MIN ? 0x1p16f : 1.0f);
+}
+
 // Scale t of the interaction kernel for length h (FP32).
 float kernel_scale(int kernel, float h)
 {
     const double hd = (double)h;
     switch (kernel) {
         case PI_KERNEL_LJ:
-        case PI_KERNEL_HIGHFLOP: return (float)std::fmin(1.0 / (hd * hd), (double)FLT_MAX);  // 1 / sigma^2, finite
+        case PI_KERNEL_HIGHFLOP: return (float)((double)lj_power(h) / (hd * hd));  // e / sigma^2
         case PI_KERNEL_LOWFLOP: return 0.f;
         default: return (float)(-1.4426950408889634 / (hd * hd));  // -log2(e) / h^2
     }
 }
 
 // The FP32 remainder of the Gaussian's FP64 scale after its FP32 value (the
-// fine Gaussian uses t + tl).
+// fine Gaussian uses t + tl); the power of two in the Lennard-Jones scale.
 float kernel_scale_lo(int kernel, float h)
 {
+    if (kernel == PI_KERNEL_LJ || kernel == PI_KERNEL_HIGHFLOP) return lj_power(h);
     if (kernel != PI_KERNEL_GAUSSIAN) return 0.f;
     const double hd = (double)h, t = -1.4426950408889634 / (hd * hd);
     return (float)(t - (double)(float)t);

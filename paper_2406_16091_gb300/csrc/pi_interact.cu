@@ -74,16 +74,21 @@ __device__ __forceinline__ float rcp_approx(float x)
 }
 
 // The Lennard-Jones kernel's s = 1 / u, u = r^2/sigma^2 + 1/100, is the
-// hardware's approximate reciprocal q of u (one ulp) and one Newton step,
-// q + q (1 - u q): half an ulp of u's reciprocal, at 3 instructions instead
-// of the correctly rounded __frcp_rn's scaling and branches, and u >= 1/100
-// needs neither.  u is cut off at LJ_FAR, far outside every cutoff that
-// leaves s^3 in FP32 (a row's sentinel slots would overflow it, and the step
-// turn infinity into NaN), where K is an exact zero.  4 (s^6 - s^3) is
-// s^3 (4 s^3 - 4), two roundings where there were three.  Measured (medians
+// hardware's approximate reciprocal q of u (within one ulp, as PTX documents
+// rcp.approx) and one Newton-Raphson step, q + q (1 - u q), within one ulp of
+// u's reciprocal again; u >= 1/100 needs no scaling.  u is cut off at LJ_FAR,
+// far outside every cutoff that leaves s^3 in FP32 (a row's sentinel slots
+// would overflow it, and the step turn infinity into NaN), where K is an
+// exact zero.  4 (s^6 - s^3) is s^3 (4 s^3 - 4), two roundings where there
+// were three.  Where 1/sigma^2 is no normal FP32 number, u carries a power of
+// two e (KParams::tl) that makes e/sigma^2 one; s^3 is then e^-3 times
+// larger, and the value's two constants take the powers back:
+// s^3 (4 e^6 s^3 - 4 e^3), with e = 1 otherwise.  Measured (medians
 // of the interaction in us, sigma^2 __frcp_rn(r^2 + sigma^2/100) / this):
 // 104 / 84 at 500,009 particles and 350 / 277 at 2 M, 8 per cell, 1008 / 786
-// at 32 per cell, 563 / 401 clustered (500,000).
+// at 32 per cell, 563 / 401 clustered (500,000).  The value's constants from
+// registers instead of immediates: 290.5 / 286.6 at 2 M and 8 per cell, 886 /
+// 874 at 32; the 168-FLOP kernel 888 / 896; shape 2 178.6 / 180.5 (500,009).
 constexpr float LJ_FAR = 1.2676506e30f;  // 2^100
 
 // Accumulators.  add(t, in) adds the term t of a candidate that passed the
@@ -130,9 +135,11 @@ struct KahanAcc {
 };
 
 // Scale of the kernel (t; for the fine Gaussian also the remainder tl of
-// the FP64 scale after t) and the opaque constants of the high-FLOP kernel.
+// the FP64 scale after t, for Lennard-Jones its power of two e), the opaque
+// constants of the high-FLOP kernel, and those of the Lennard-Jones value:
+// e/100, 4 e^6 and -4 e^3 (exact but for 1/100).
 struct KParams {
-    float t, tl, one, zero;
+    float t, tl, one, zero, lj_soft, lj_six, lj_three;
 };
 
 // s + e = a + b exactly (Knuth's two-sum, six rounded operations).
@@ -175,7 +182,7 @@ __device__ __forceinline__ float gauss_fine(float dx, float dy, float dz, float 
 
 // Value of the interaction kernel for one pair inside the cutoff at FP32
 // offset (dx, dy, dz), r2 the frozen FP32 squared distance; kp.t is the
-// system's scale (Gaussian: -log2(e)/h^2; Lennard-Jones: 1/sigma^2).
+// system's scale (Gaussian: -log2(e)/h^2; Lennard-Jones: e/sigma^2).
 template <int KERNEL>
 __device__ __forceinline__ float kernel_value(float dx, float dy, float dz, float r2, const KParams& kp)
 {
@@ -186,11 +193,11 @@ __device__ __forceinline__ float kernel_value(float dx, float dy, float dz, floa
     } else if constexpr (KERNEL == KERNEL_LOWFLOP) {
         return 1.0f;
     } else {
-        const float u = fminf(__fmaf_rn(r2, kp.t, 0.01f), LJ_FAR);
+        const float u = fminf(__fmaf_rn(r2, kp.t, kp.lj_soft), LJ_FAR);
         const float q = rcp_approx(u);
         const float sr = __fmaf_rn(q, __fmaf_rn(-u, q, 1.0f), q);
         const float s3 = __fmul_rn(__fmul_rn(sr, sr), sr);
-        float K = __fmul_rn(s3, __fmaf_rn(s3, 4.0f, -4.0f));
+        float K = __fmul_rn(s3, __fmaf_rn(s3, kp.lj_six, kp.lj_three));
         if constexpr (KERNEL == KERNEL_HIGHFLOP) {
 #pragma unroll
             for (int i = 0; i < 75; ++i) K = __fmaf_rn(K, kp.one, kp.zero);
@@ -200,11 +207,12 @@ __device__ __forceinline__ float kernel_value(float dx, float dy, float dz, floa
 }
 
 // The kernel parameters of system sid: kscale holds the S scales, then the
-// S remainders of the fine Gaussian.
+// S remainders of the fine Gaussian, or powers of two of Lennard-Jones.
 __device__ __forceinline__ KParams kparams(const InteractArgs& a, int sid)
 {
-    return a.kscale ? KParams{a.kscale[sid], a.kscale[a.sy.S + sid], a.one, a.zero}
-                    : KParams{a.kscale0, a.kscale0_lo, a.one, a.zero};
+    const float t = a.kscale ? a.kscale[sid] : a.kscale0, tl = a.kscale ? a.kscale[a.sy.S + sid] : a.kscale0_lo;
+    const float e3 = tl * tl * tl;
+    return KParams{t, tl, a.one, a.zero, 0.01f * tl, 4.0f * e3 * e3, -4.0f * e3};
 }
 
 // Every path excludes the self pair by identity (the source's stable slot
@@ -799,12 +807,13 @@ __device__ __forceinline__ float2 packed_value(float2 dx, float2 dy, float2 dz, 
         K = m;
     } else {
         // kernel_value's Lennard-Jones steps, element by element
-        const float2 w = __ffma2_rn(r2, ks, make_float2(0.01f, 0.01f));
+        const float2 w = __ffma2_rn(r2, ks, make_float2(kp.lj_soft, kp.lj_soft));
         const float2 u = make_float2(fminf(w.x, LJ_FAR), fminf(w.y, LJ_FAR));
         const float2 q = make_float2(rcp_approx(u.x), rcp_approx(u.y));
         const float2 sr = __ffma2_rn(q, __ffma2_rn(make_float2(-u.x, -u.y), q, make_float2(1.f, 1.f)), q);
         const float2 s3 = __fmul2_rn(__fmul2_rn(sr, sr), sr);
-        float2 e = __fmul2_rn(s3, __ffma2_rn(s3, make_float2(4.f, 4.f), make_float2(-4.f, -4.f)));
+        float2 e = __fmul2_rn(s3, __ffma2_rn(s3, make_float2(kp.lj_six, kp.lj_six),
+                                             make_float2(kp.lj_three, kp.lj_three)));
         if constexpr (KERNEL == KERNEL_HIGHFLOP) {
             const float2 one = make_float2(kp.one, kp.one), zero = make_float2(kp.zero, kp.zero);
 #pragma unroll
@@ -1323,7 +1332,7 @@ __device__ void ws_consumer(const InteractArgs& a, WsSmem<T>& sm, unsigned tid, 
                   ng = st.ngroups;
         const uint32_t tb = st.tb;
         const int first = mode == 0 ? p.sbeg[4] + (int)(tb - p.gbeg[4]) : (int)tb;
-        const KParams kp{st.t, 0.f, a.one, a.zero};  // the fine Gaussian never runs here
+        const KParams kp{st.t, 0.f, a.one, a.zero, 0.f, 0.f, 0.f};  // only the plain Gaussian runs here
         for (;;) {
             int g = 0;
             if (lane == 0) g = atomicAdd(&st.next_group, 1);

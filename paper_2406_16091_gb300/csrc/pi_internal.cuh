@@ -491,8 +491,8 @@ struct InteractArgs {
     uint32_t np;            // entries of P: n plus ROW_PADS per X-row
     uint32_t work;          // work items (X-row segments) of all systems
     const float* kscale;    // [2S]: scale t of system s at [s] (Gaussian K = 2^(r2 t), t =
-                            // -log2(e)/h^2 in FP32; Lennard-Jones 1/sigma^2), the FP32
-                            // remainder of the FP64 scale at [S + s] (fine Gaussian)
+                            // -log2(e)/h^2 in FP32; Lennard-Jones e/sigma^2), at [S + s]
+                            // the FP32 remainder of the FP64 scale (fine Gaussian) or e
     float kscale0;          // the scale and remainder when S == 1 (kscale may then be null)
     float kscale0_lo;
     int kernel;             // KERNEL_*
