@@ -13,6 +13,8 @@
 #include <new>
 #include <vector>
 
+#include <cuda.h>
+
 #include "pi.h"
 #include "pi_internal.cuh"
 
@@ -556,15 +558,38 @@ static bool record_stream(cudaStream_t s, unsigned long long* stream, unsigned l
     return e == cudaSuccess && cap != cudaStreamCaptureStatusInvalidated;
 }
 
-// Whether ptr is memory that was allocated on the context's device.
-static bool own_memory(const pi_ctx* ctx, const void* ptr)
+// The driver's pointer query (one call for all the attributes; the runtime's
+// does not tell an allocation's extent), or null.
+static decltype(&cuPointerGetAttributes) pointer_query()
 {
-    cudaPointerAttributes at{};
-    if (cudaPointerGetAttributes(&at, ptr) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return false;
-    }
-    return at.type == cudaMemoryTypeDevice && at.device == ctx->device;
+    static const auto query = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 7000, cudaEnableDefault, &found) !=
+            cudaSuccess)
+            (void)cudaGetLastError();
+        return found == cudaDriverEntryPointSuccess ? (decltype(&cuPointerGetAttributes))f : nullptr;
+    }();
+    return query;
+}
+
+// Whether the `bytes` bytes from ptr on lie in one allocation on the context's
+// device (which is current): what a kernel may write as a memory copy would.
+static bool own_memory(const pi_ctx* ctx, const void* ptr, size_t bytes)
+{
+    const auto query = pointer_query();
+    if (!query) return false;
+    unsigned type = 0, managed = 0;
+    int device = -1;
+    CUdeviceptr start = 0;
+    size_t size = 0;
+    CUpointer_attribute what[5] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                                   CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                   CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void* into[5] = {&type, &managed, &device, &start, &size};
+    if (query(5, what, into, (CUdeviceptr)ptr) != CUDA_SUCCESS) return false;
+    const size_t at = (size_t)((CUdeviceptr)ptr - start);
+    return type == CU_MEMORYTYPE_DEVICE && !managed && device == ctx->device && at <= size && bytes <= size - at;
 }
 
 pi_status pi_copy_binned(const pi_ctx* ctx, uint32_t* counts, uint32_t* offsets, uint32_t* perm,
@@ -584,12 +609,13 @@ pi_status pi_copy_binned(const pi_ctx* ctx, uint32_t* counts, uint32_t* offsets,
     // particles, 35.1 / 33.9 at 32,768, 441 / 437 for 64 systems).  It writes
     // by plain stores and in no order, so memory copies, one after the other,
     // stay for destinations that are not word-aligned, not memory of this
-    // device (host or another device's memory), or that overlap.
+    // device (host or another device's memory), that overlap, or that end
+    // before the array does (which a memory copy refuses).
     pi::CopyArgs c{};
     bool plain = true;
     for (int k = 0; k < 6; ++k) {
         if (!dst[k] || words[k] == 0) continue;
-        plain = plain && (uintptr_t)dst[k] % 4 == 0 && own_memory(ctx, dst[k]);
+        plain = plain && (uintptr_t)dst[k] % 4 == 0 && own_memory(ctx, dst[k], words[k] * 4);
         for (int j = 0; j < c.count; ++j)
             plain = plain && ((uint32_t*)dst[k] + words[k] <= c.dst[j] || c.dst[j] + c.words[j] <= (uint32_t*)dst[k]);
         c.src[c.count] = (const uint32_t*)src[k];
