@@ -310,8 +310,8 @@ pi_status pi_batch_interact(pi_ctx* ctx, const float* h, float* S, float* Vx, fl
  * algorithm (PI_OPT_TILE 0..6), then with PI_ALGO_PPNL, and -- for a batch
  * context -- with a shape per occupancy regime: the systems are grouped by
  * mean particles per cell (below 4, 4 to 8, 8 and more), each group is
- * timed alone with shapes 5 and 6 and takes the faster, and the resulting
- * per-system plan (pi_batch_set_tiles) is timed as a whole.  The candidate
+ * timed with shapes 5 and 6 while the others run shape 5 and takes the
+ * faster, and the resulting per-system plan (pi_batch_set_tiles) is timed.  The candidate
  * with the smallest median time is kept for later calls (PI_OPT_ALGO,
  * PI_OPT_TILE or the per-system plan); *chosen receives its index (0..6 =
  * tile shape, 7 = PI_ALGO_PPNL, 8 = the per-regime plan) and ms[9] the

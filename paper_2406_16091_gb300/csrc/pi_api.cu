@@ -95,7 +95,7 @@ struct pi_ctx {
     size_t mat_cap;                 // entries of mat (mat_base has one more)
 
     // per-system tile shapes of a batch (empty: every system runs `tile`);
-    // entries 5 or 6, or 0 for a system left out (autotuner trials only)
+    // entries 5 or 6
     std::vector<int> sys_tile;
     // device range lists of the per-system shapes: [0, 2S) the ranges of
     // shape 5, [2S, 4S) of shape 6, [4S, 5S) and [5S, 6S) their first blocks
@@ -897,6 +897,19 @@ pi_status launch_plan(pi_ctx* ctx, pi::InteractArgs a, bool kahan, cudaStream_t 
     return PI_OK;
 }
 
+// The kernel that a launch runs: the Gaussian with the compensated exponent
+// where some system's kernel is short next to its cutoff (r_c^2 / h^2 above
+// FINE_GAUSS_RATIO).
+int launched_kernel(const pi_ctx* ctx, const float* h)
+{
+    if (ctx->kernel == PI_KERNEL_GAUSSIAN)
+        for (int s = 0; s < ctx->S; ++s) {
+            const double r = (double)ctx->rc[s] / (double)h[s];
+            if (r * r > pi::FINE_GAUSS_RATIO) return pi::KERNEL_GAUSSIAN_FINE;
+        }
+    return ctx->kernel;
+}
+
 // Whether shape 5 takes one target per thread (k_interact_direct1) instead
 // of two.  Medians of the interaction in us, two targets / one (particles,
 // mean per cell):
@@ -945,10 +958,7 @@ bool records_pay(const pi_ctx* ctx, const pi::InteractArgs& a)
 {
     if (ctx->algo == PI_ALGO_PPNL || ctx->precision == PI_PREC_KAHAN || ctx->count_evals || a.one_target) return false;
     if (a.kernel != pi::KERNEL_GAUSSIAN && a.kernel != pi::KERNEL_LOWFLOP && a.kernel != pi::KERNEL_LJ) return false;
-    // every target of the launch must be written: direct shapes, no system left out
-    if (ctx->sys_tile.empty() ? (ctx->tile >= 0 && ctx->tile < pi::DEFAULT_TILE)
-                              : std::find(ctx->sys_tile.begin(), ctx->sys_tile.end(), 0) != ctx->sys_tile.end())
-        return false;
+    if (ctx->sys_tile.empty() && ctx->tile >= 0 && ctx->tile < pi::DEFAULT_TILE) return false;  // the staged shapes
     const double n = (double)ctx->n, C = (double)ctx->C;
     if (ctx->n < UNPERMUTE_MIN) return false;
     if (n < 8 * C) return n < 4 * C || n >= 1.5 * (double)UNPERMUTE_MIN;
@@ -1002,15 +1012,8 @@ pi_status pi_batch_interact(pi_ctx* ctx, const float* h, float* S, float* Vx, fl
     a.work = ctx->work;
     a.one = 1.0f;
     a.zero = 0.0f;
-    // the Gaussian with the compensated exponent where some system's kernel
-    // is short next to its cutoff (r_c^2 / h^2 above FINE_GAUSS_RATIO)
-    bool fine = false;
-    if (ctx->kernel == PI_KERNEL_GAUSSIAN)
-        for (int s = 0; s < ctx->S; ++s) {
-            const double r = (double)ctx->rc[s] / (double)h[s];
-            fine = fine || r * r > pi::FINE_GAUSS_RATIO;
-        }
-    a.kernel = fine ? pi::KERNEL_GAUSSIAN_FINE : ctx->kernel;
+    a.kernel = launched_kernel(ctx, h);
+    const bool fine = a.kernel == pi::KERNEL_GAUSSIAN_FINE;
     if (ctx->S == 1) {
         a.kscale = nullptr;
         a.kscale0 = kernel_scale(ctx->kernel, h[0]);
@@ -1131,7 +1134,7 @@ pi_status pi_autotune(pi_ctx* ctx, const float* h, float* S, float* Vx, float* V
     // candidates: every tile shape of the tiled algorithm, then Alg. 1, then
     // (batches) a shape per occupancy regime
     constexpr int PPNL = pi::NUM_TILES, REGIMES = pi::NUM_TILES + 1;
-    float best = 0.f;
+    float best = 0.f, shape5 = 0.f;
     int best_c = -1;
     ctx->sys_tile.clear();
     for (int t = 0; t <= PPNL && result == PI_OK; ++t) {
@@ -1140,6 +1143,7 @@ pi_status pi_autotune(pi_ctx* ctx, const float* h, float* S, float* Vx, float* V
         float med = 0.f;
         if (!median_ms(med)) break;
         if (ms) ms[t] = med;
+        if (t == 5) shape5 = med;
         if (best_c < 0 || med < best) {
             best = med;
             best_c = t;
@@ -1148,26 +1152,29 @@ pi_status pi_autotune(pi_ctx* ctx, const float* h, float* S, float* Vx, float* V
     if (ms) ms[REGIMES] = 0.f;
     std::vector<int> plan;
     if (result == PI_OK && ctx->S > 1) {
-        // per regime, the faster direct shape on its systems alone
+        // per regime, the faster direct shape on its systems while the others
+        // run shape 5: whole plans, whose outputs take the way that the
+        // chosen plan's will (records or straight, see records_pay)
         ctx->algo = PI_ALGO_TILED;
-        plan.assign(ctx->S, 0);
+        plan.assign(ctx->S, 5);
+        float all5 = shape5;  // (a plan's shape 5 takes two targets per thread)
+        ctx->sys_tile = plan;
+        if (one_target_form(ctx, launched_kernel(ctx, h))) median_ms(all5);
         for (int g = 0; g < 3 && result == PI_OK; ++g) {
-            std::vector<int> trial(ctx->S, 0);
+            std::vector<int> trial(ctx->S, 5);
             bool any = false;
             for (int s = 0; s < ctx->S; ++s)
-                if (occupancy_regime(ctx, s) == g && ctx->pbase_h[s + 1] > ctx->pbase_h[s]) any = true;
+                if (occupancy_regime(ctx, s) == g) {
+                    trial[s] = 6;
+                    any = any || ctx->pbase_h[s + 1] > ctx->pbase_h[s];
+                }
             if (!any) continue;
-            float tm[2] = {0.f, 0.f};
-            for (int k = 0; k < 2 && result == PI_OK; ++k) {
-                for (int s = 0; s < ctx->S; ++s) trial[s] = occupancy_regime(ctx, s) == g ? 5 + k : 0;
-                ctx->sys_tile = trial;
-                median_ms(tm[k]);
-            }
-            for (int s = 0; s < ctx->S; ++s)
-                if (occupancy_regime(ctx, s) == g) plan[s] = tm[1] < tm[0] ? 6 : 5;
+            float with6 = 0.f;
+            ctx->sys_tile = trial;
+            if (median_ms(with6) && with6 < all5)
+                for (int s = 0; s < ctx->S; ++s)
+                    if (trial[s] == 6) plan[s] = 6;
         }
-        for (int s = 0; s < ctx->S; ++s)
-            if (plan[s] == 0) plan[s] = 5;  // systems without particles
         float med = 0.f;
         ctx->sys_tile = plan;
         if (result == PI_OK && median_ms(med)) {
@@ -1194,8 +1201,7 @@ pi_status pi_autotune(pi_ctx* ctx, const float* h, float* S, float* Vx, float* V
     else
         ctx->sys_tile.clear();
     if (chosen) *chosen = best_c;
-    // the outputs of the chosen configuration (the last trial may have left
-    // some systems out)
+    // the outputs of the chosen configuration
     return pi_batch_interact(ctx, h, S, Vx, Vy, Vz, nbr, out_order, stream);
 }
 

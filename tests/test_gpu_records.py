@@ -161,3 +161,28 @@ def test_batch_with_a_plan_of_both_shapes():
             assert same(torch, r, results[0])
     finally:
         B.pi_destroy(ctx)
+
+
+def test_autotuned_plans_are_timed_on_the_way_they_run():
+    # a batch over three occupancy regimes whose plan writes records: so do the
+    # trials of the regimes, each interaction one launch more than sorted
+    torch = pytest.importorskip("torch")
+    s = torch.cuda.current_stream()
+    ns, rcs, reps = [600001, 600000, 300000], [W.rc_for_cells(c) for c in (100, 50, 30)], 3
+    ctx = B.pi_batch_create([BOX] * 3, rcs, ns)
+    try:
+        p = [W.uniform(k, 7 + i) for i, k in enumerate(ns)]
+        pos = [torch.from_numpy(np.concatenate([q[d] for q in p])).cuda() for d in range(3)]
+        h, n, launches = [r / 2 for r in rcs], sum(ns), []
+        _, out = outputs(torch, n)
+        for order in (B.PI_ORDER_SORTED, B.PI_ORDER_ORIGINAL):
+            B.pi_batch_set_tiles(ctx, None)
+            B.pi_batch_bin(ctx, *pos, ns, s)
+            before = B.pi_launch_count(ctx)
+            B.pi_autotune(ctx, h, *out, order, reps, s)
+            launches.append(B.pi_launch_count(ctx) - before)
+        # shapes 5 and 6, three regimes and the resulting plan write records; that plan may take one launch (and one
+        # that writes its ranges) fewer in this order than in the other
+        assert launches[1] - launches[0] >= (reps + 1) * (6 - 1) - 2
+    finally:
+        B.pi_destroy(ctx)
