@@ -535,8 +535,9 @@ pi_status pi_binned(const pi_ctx* ctx, const uint32_t** counts, const uint32_t**
 }
 
 // Input-order outputs go through the binning's records (launch_unpermute)
-// from this many particles on (see records_pay).
-constexpr int64_t UNPERMUTE_MIN = 1000000;
+// from this many particles on, or this many at 8 and more per cell (see
+// records_pay).
+constexpr int64_t UNPERMUTE_MIN = 1000000, UNPERMUTE_MIN_DENSE = 5500000;
 
 // The identity of a stream and of the capture it is in (0: none); false if
 // either is not to be had.  The records belong to the stream, and capture, of
@@ -940,20 +941,30 @@ bool one_target_form(const pi_ctx* ctx, int kernel)
 // straight to the arrays: in the two- and four-target direct kernels with
 // plain Gaussian, low-FLOP or Lennard-Jones sums (recorded_form; the
 // compensated sums hide the words throughout: 8.4 M at 8 2010 / 2036, 16.8 M
-// 4071 / 4137).  The extra pass costs about
-// 5 us per million particles.  Against it stand the scattered words, which a
-// long evaluation hides as long as the L2 holds the arrays.  Medians of a
-// step in us, straight / records (particles, mean per cell):
-//   - two targets per thread: 600,000 at 1 75.6 / 77.7 (an earlier k_unpermute),
-//     1 M at 1 121.8 / 114.4 and at 4 140 / 136, 1.5 M at 2 182 / 169, 2 M at
-//     1 251 / 230 and at 6 319 / 303, 16.8 M at 1 3294 / 2018, clustered 2 M
-//     at 1 516 / 514 and at 2 810 / 797;
-//   - four targets, whose evaluation is longer, from n = 65536 q^2 at q per
-//     cell: 2 M at 8 324 / 335, 3 M at 8 454 / 470, 4.2 M at 8 678 / 652, 8.4 M
-//     at 8 1540 / 1334, 4.2 M at 12 756 / 786, 8.4 M at 12 1593 / 1576, 16.8 M
-//     at 16 3697 / 3710 and at 32 5704 / 5909;
-//   - Lennard-Jones likewise: 1 M at 1 128 / 125, 2 M at 4 303 / 300, 8.4 M
-//     at 8 1616 / 1533, 16.8 M at 2 3713 / 2196 and at 16 4666 / 4605.
+// 4071 / 4137).  The extra pass costs about 7.7 us per million particles out
+// of DRAM (52 bytes each), less while the records are in the L2.  Against it
+// stand the scattered words, which a long evaluation hides as long as the L2
+// holds the arrays: past 6 M particles they take 130 to 175 ns per thousand
+// whatever the evaluation.  Medians of a step (binning included) in us,
+// straight / records (particles, mean per cell):
+//   - below 8 per cell (two targets per thread): 600,000 at 1 82.6 / 81.6, 1 M
+//     at 1 127.6 / 122.5, 1.5 M at 2 187 / 173 and at 6 236 / 225, 2 M at 1
+//     250 / 230 and at 6 322 / 308, 4.2 M at 4 548 / 519, clustered 2 M at 1
+//     522 / 518 and at 2 812 / 800.  (From 4 per cell the line is 1.5 M,
+//     though 1 M at 4 takes 145 / 140.)
+//   - from 8 on (four targets, whose evaluation is longer): the more per
+//     cell, the larger n has to be, n = 65536 q^2 at q per cell, and 5.5 M at
+//     the least.  4.5 M at 8.5 699 / 721, 5.0 M at 8.7 791 / 809, 5.5 M at 8.7
+//     885 / 885 and at 9.6 918 / 925, 6.5 M at 8.6 1096 / 1046, 9 M at 11.6
+//     1723 / 1652, 12 M at 12 2457 / 2252, 14.5 M at 15.9 3154 / 3169, 16.8 M at
+//     8 3630 / 2660 and at 15.8 3697 / 3662.  (One GPU of several wrote the
+//     words faster: there 12 M at 12 took 2200 / 2227, 16.8 M at 8 3036 / 2613
+//     and at 15.8 3540 / 3641.)
+//   - Lennard-Jones, two targets throughout: 1 M at 1 134 / 130 and at 2.9
+//     144 / 145, 1.5 M at 4 224 / 221, 2 M at 4 307 / 304 and at 7 351 / 353,
+//     4 M at 7 691 / 695, 16.8 M at 2 3041 / 2155; 4.2 M at 8 756 / 766, 5.0 M at
+//     8.7 953 / 959, 5.5 M at 8.7 1051 / 1049, 6.5 M at 9.9 1344 / 1326, 9 M at
+//     12 2066 / 2054, 16.8 M at 15.8 4621 / 4607.
 bool records_pay(const pi_ctx* ctx, const pi::InteractArgs& a)
 {
     if (ctx->algo == PI_ALGO_PPNL || ctx->precision == PI_PREC_KAHAN || ctx->count_evals || a.one_target) return false;
@@ -962,7 +973,7 @@ bool records_pay(const pi_ctx* ctx, const pi::InteractArgs& a)
     const double n = (double)ctx->n, C = (double)ctx->C;
     if (ctx->n < UNPERMUTE_MIN) return false;
     if (n < 8 * C) return n < 4 * C || n >= 1.5 * (double)UNPERMUTE_MIN;
-    return C * C >= 65536.0 * n;
+    return ctx->n >= UNPERMUTE_MIN_DENSE && C * C >= 65536.0 * n;
 }
 
 // Occupancy regimes of the per-system autotuning: mean particles per cell

@@ -186,3 +186,22 @@ def test_autotuned_plans_are_timed_on_the_way_they_run():
         assert launches[1] - launches[0] >= (reps + 1) * (6 - 1) - 2
     finally:
         B.pi_destroy(ctx)
+
+
+@pytest.mark.parametrize("n,cells,launched", [(5000001, 84, 1), (5499999, 87, 1), (5500000, 87, 2), (5500000, 83, 1)])
+@pytest.mark.parametrize("kernel", [B.PI_KERNEL_GAUSSIAN, B.PI_KERNEL_LJ])
+def test_line_from_eight_per_cell(n, cells, launched, kernel):
+    torch = pytest.importorskip("torch")
+    s = torch.cuda.current_stream()
+    ctx, h, pos = setup(torch, n, cells, kernel)
+    try:
+        B.pi_bin(ctx, *pos, n, s)
+        want = in_order(torch, ctx, h, n, s)
+        _, out = outputs(torch, n)
+        before = B.pi_launch_count(ctx)
+        B.pi_interact(ctx, h, *out, B.PI_ORDER_ORIGINAL, s)
+        assert B.pi_launch_count(ctx) - before == launched
+        B.pi_sync_status(ctx, s)
+        assert same(torch, out, want)
+    finally:
+        B.pi_destroy(ctx)
