@@ -912,29 +912,37 @@ int launched_kernel(const pi_ctx* ctx, const float* h)
 }
 
 // Whether shape 5 takes one target per thread (k_interact_direct1) instead
-// of two.  Medians of the interaction in us, two targets / one (particles,
-// mean per cell):
+// of two.  Medians of the interaction (four in a row) in us, two targets /
+// one (particles, mean per cell):
 //   - few particles: one thread's chain of trips sets the time, and one
-//     target halves it, up to about 256 threads per SM (Gaussian: 1,531 at 6
-//     18.4 / 14.4, 10,000 at 8 22.5 / 16.4, 32,768 at 8 20.5 / 18.4, 65,536
-//     at 8 22.5 / 24.6; Lennard-Jones: 30,000 clustered 41.0 / 30.7, 60,000
-//     at 8 24 / 22.5, 131,072 at 8 34.8 / 34.8, 100,000 dense clusters 207 /
-//     299);
+//     target halves it, up to 256 threads per SM (Gaussian: 1,531 at 6
+//     13.0 / 10.1, 10,000 at 8 15.3 / 11.2, 38,912 at 8 16.3 / 13.7, 65,536
+//     at 8 18.3 / 18.3; Lennard-Jones: 30,000 at 8 17.8 / 13.7, 60,000
+//     at 8 19.4 / 17.3, 131,072 at 8 29.6 / 31.1, dense clusters 38,000 87 /
+//     83 and 100,000 208 / 307, hence no higher line);
 //   - the 168-FLOP kernel spends most on each evaluation, and one target
-//     has fewer of them: 465 / 375 and 975 / 922 (2 M at 2 and 8), dense
-//     clusters 2540 / 2132 (300,000 at 16);
-//   - the compensated exponent likewise below 16 per cell: 242 / 213, 473 /
-//     469 and 1436 / 1464 (2 M at 2, 8 and 32), with compensated sums 180 /
-//     162 (500,000 at 8);
-//   - the compensated sums below 6 per cell: 211 / 195, 270 / 258 and 336 /
-//     322 (2 M at 2, 4 and 6), clustered 618 / 584 (1 M at 2) and 881 / 997
-//     (300,000 at 16: cells of more than 255 take their exact windows).
+//     has fewer of them: 454 / 368, 969 / 897 and 3206 / 3004 (2 M at 2, 8 and
+//     32), dense clusters 2125 / 1833 (300,000 at 16);
+//   - the compensated exponent likewise, against which stands that a source
+//     read feeds one target instead of two: below 9 per cell 243 / 219, 412 / 406, 491 /
+//     490, 526 / 526 and 662 / 668 (2 M at 2, 6, 8, 9 and 12), 963 / 964 and
+//     1337 / 1353 (4.2 M at 8 and 12); below 16 up to 6,500 particles per SM,
+//     127 / 121 and 225 / 219 (500,000 at 8 and 16), 320 / 318 and 401 / 402
+//     (1 M at 12 and 16), clustered 1067 / 1036 (300,000 at 15), and with
+//     compensated sums, 175 / 159 and 313 / 292 (500,000 at 8 and 16), 1116 /
+//     1072 (2 M at 15);
+//   - the compensated sums below 6 per cell: 213 / 199, 276 / 262 and 349 /
+//     334 (2 M at 2, 4 and 6), clustered 669 / 571 (1 M at 2); at 8 416 / 398
+//     still, but layouts of a higher mean may hold cells of more than 255,
+//     which take their exact windows: 867 / 993 (300,000 clustered at 16).
 bool one_target_form(const pi_ctx* ctx, int kernel)
 {
     if (ctx->n <= (int64_t)ctx->num_sms * 256) return true;
     if (kernel == pi::KERNEL_HIGHFLOP) return true;
-    if (kernel == pi::KERNEL_GAUSSIAN_FINE) return ctx->n < 16 * ctx->C;
-    return ctx->precision == PI_PREC_KAHAN && ctx->n < 6 * ctx->C;
+    const bool kahan = ctx->precision == PI_PREC_KAHAN;
+    if (kernel == pi::KERNEL_GAUSSIAN_FINE)
+        return ctx->n < (kahan || ctx->n <= (int64_t)ctx->num_sms * 6500 ? 16 : 9) * ctx->C;
+    return kahan && ctx->n < 6 * ctx->C;
 }
 
 // Whether input-order outputs go through records and k_unpermute instead of
@@ -1079,9 +1087,10 @@ pi_status pi_batch_interact(pi_ctx* ctx, const float* h, float* S, float* Vx, fl
         // four-target grid has at least 480 threads per SM, three quarters of
         // a wave of 5 CTAs of 128; two otherwise: a smaller grid leaves SMs
         // idle and each thread twice the work.  Medians in us, two / four
-        // targets: 200,000 at 10 per cell 36.8 / 38.8, 262,144 at 8 38.8 /
-        // 41.4, 300,000 at 10 49.6 / 47.5 and at 32 119.7 / 109.0, clustered
-        // 300,000 at 8 389 / 357 and at 16 531 / 462.  The four-target
+        // targets: 200,000 at 10 per cell 36.8 / 38.8, 262,144 at 8 38.3 /
+        // 41.4, 300,000 at 10 49.1 / 48.0 and at 32 120 / 110, clustered
+        // 300,000 at 8 391 / 357 and at 16 529 / 463, 2 M at 6 197 / 201, at 7
+        // 213 / 214, at 8 233 / 230 and at 32 739 / 637.  The four-target
         // Lennard-Jones and 168-FLOP forms (slower at 8 per cell, no faster
         // at 32) and the compensated sums keep all their registers and run
         // fewer warps
