@@ -13,7 +13,10 @@ from gpu_harness import check_interaction, oracle_run, run_gpu
 
 pytestmark = pytest.mark.gpu
 
-SMS = 152  # of one GB300; the sizes below lie on both sides of the line there
+
+def _sms():
+    torch = pytest.importorskip("torch")
+    return torch.cuda.get_device_properties(0).multi_processor_count
 
 
 def _uniform(n, ppc, seed=31):
@@ -35,9 +38,9 @@ CASES = {
     "ragged_4099": lambda: _uniform(4099, 6),
     "long_rows": lambda: (*W.uniform(5001, 6, (0, 0, 0), (3.0, 0.04, 0.04)), (0, 0, 0), (3.0, 0.04, 0.04), 0.01),
     "dense": lambda: _dense(6001),
-    "line_256": lambda: _uniform(SMS * 256, 3),
-    "past_256": lambda: _uniform(SMS * 256 + 1, 5),
-    "larger": lambda: _uniform(SMS * 1024 + 1, 3),
+    "line_256": lambda: _uniform(_sms() * 256, 3),
+    "past_256": lambda: _uniform(_sms() * 256 + 1, 5),
+    "larger": lambda: _uniform(_sms() * 1024 + 1, 3),
 }
 FORMS = [(B.PI_KERNEL_GAUSSIAN, B.PI_PREC_FP32, 2), (B.PI_KERNEL_GAUSSIAN, B.PI_PREC_KAHAN, 2),
          (B.PI_KERNEL_GAUSSIAN, B.PI_PREC_FP32, 8), (B.PI_KERNEL_LJ, B.PI_PREC_FP32, 2),
@@ -60,3 +63,15 @@ def test_one_target_form_matches_the_other_shapes(name, kern, prec, hdiv):
     if name in ("one", "ragged_4099", "long_rows"):
         _, r = oracle_run(x, y, z, lo, hi, rc, h, kern)
         check_interaction(runs[0], r, rc=rc)
+
+
+@pytest.mark.parametrize("past", [0, 1])
+@pytest.mark.parametrize("prec", [B.PI_PREC_FP32, B.PI_PREC_KAHAN])
+def test_compensated_exponent_on_both_sides_of_its_line(past, prec):
+    # 9 to 16 per cell: one target per thread up to 6,500 particles per SM, and with compensated sums
+    x, y, z, lo, hi, rc = _uniform(_sms() * 6500 + past, 12)
+    runs = [run_gpu(x, y, z, lo, hi, rc, rc / 8, tile=t, precision=prec, binned=False) for t in (5, 6)]
+    for g in runs:
+        assert g["status"] == B.PI_OK
+    for k in ("S", "Vx", "Vy", "Vz", "nbr"):
+        assert np.array_equal(runs[0][k].view(np.uint32), runs[1][k].view(np.uint32)), k

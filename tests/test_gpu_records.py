@@ -1,7 +1,7 @@
 """Input-order outputs of large systems, written as records and copied to the
 arrays by a second kernel: bitwise the sorted-order outputs in input order, at
-the rule's edges, for both direct shapes, without neighbour counts, at odd
-alignments, and nothing written beside the arrays.  Calls that may overlap
+the rule's edges, for both direct shapes, in dense cells, without neighbour
+counts, at odd alignments, and nothing written beside the arrays.  Calls that may overlap
 (another stream, an interaction captured alone) write straight to the arrays;
 the launch counts tell the two ways apart."""
 import numpy as np
@@ -42,6 +42,18 @@ def in_order(torch, ctx, h, n, s):
     return want
 
 
+def clustered(n, cells):
+    """Uniform but for a tight cluster of 6,000 at each of two places: cells of
+    more than 255, whose targets take exact window bounds."""
+    x = np.stack(W.uniform(n, 5), 1)
+    rng = np.random.default_rng(9)
+    for k, c in enumerate(((0.31, 0.42, 0.77), (0.8, 0.1, 0.25))):
+        x[k * 6000:(k + 1) * 6000] = np.asarray(c) + 0.6 / cells * rng.standard_normal((6000, 3))
+    x = np.clip(x, 0, np.nextafter(np.float32(1), np.float32(0))).astype(np.float32)
+    x = x[rng.permutation(n)]
+    return [np.ascontiguousarray(x[:, d]) for d in range(3)]
+
+
 def same(torch, a, b):
     return all(torch.equal(x.view(torch.int32), y.view(torch.int32)) for x, y in zip(a, b))
 
@@ -69,6 +81,26 @@ def test_records_equal_sorted_outputs(n, cells, records, kernel, tile, shift, co
         for w in whole[:used]:
             assert bool((w[:shift] == -7).all()) and bool((w[shift + n:] == -7).all())
         assert counts or bool((whole[4] == -7).all())
+    finally:
+        B.pi_destroy(ctx)
+
+
+@pytest.mark.parametrize("kernel", [B.PI_KERNEL_GAUSSIAN, B.PI_KERNEL_LOWFLOP, B.PI_KERNEL_LJ])
+@pytest.mark.parametrize("tile", [5, 6])
+def test_records_of_dense_cells(kernel, tile):
+    torch = pytest.importorskip("torch")
+    n, cells, s = EDGE + 17, 80, torch.cuda.current_stream()
+    ctx, h, _ = setup(torch, n, cells, kernel, tile)
+    try:
+        pos = [torch.from_numpy(a).cuda() for a in clustered(n, cells)]
+        B.pi_bin(ctx, *pos, n, s)
+        want = in_order(torch, ctx, h, n, s)
+        _, out = outputs(torch, n)
+        before = B.pi_launch_count(ctx)
+        B.pi_interact(ctx, h, *out, B.PI_ORDER_ORIGINAL, s)
+        assert B.pi_launch_count(ctx) - before == 2
+        assert B.pi_sync_status(ctx, s)[1] > 255
+        assert same(torch, out, want)
     finally:
         B.pi_destroy(ctx)
 

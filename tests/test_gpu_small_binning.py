@@ -1,7 +1,7 @@
 """The one-launch binning of small systems (k_bin_small: up to 4,096
 particles in up to 4,096 cells) against the oracle, at the edges of its
-range and just past them, with empty and dense cells, after an error, and on
-a context re-targeted from a larger grid."""
+range and just past them, with empty and dense cells, after an error, captured
+in a graph, and on a context re-targeted from a larger grid."""
 import numpy as np
 import pytest
 
@@ -9,7 +9,7 @@ import oracle
 from paper_2406_16091_gb300 import binding as B
 from paper_2406_16091_gb300 import workloads as W
 
-from gpu_harness import check_binning, check_interaction, oracle_run, run_gpu
+from gpu_harness import TOL, check_binning, check_interaction, oracle_run, run_gpu
 
 pytestmark = pytest.mark.gpu
 
@@ -35,16 +35,14 @@ GRIDS = {
 @pytest.mark.parametrize("grid", list(GRIDS))
 def test_small_binning_matches_the_oracle(grid, n):
     lo, hi, rc = GRIDS[grid]
-    if grid in ("one_cell", "27_cells"):
-        n = min(n, 4097)  # thousands of mutual neighbours
     x, y, z = W.uniform(n, 100 + n, lo, hi)
     b, r = oracle_run(x, y, z, lo, hi, rc, rc / 2)
     g = run_gpu(x, y, z, lo, hi, rc, rc / 2, repeat=2)
     check_binning(g, b)
-    if n <= 4097 and grid not in ("one_cell", "27_cells"):
-        check_interaction(g, r)
-    else:
-        assert np.array_equal(g["nbr"], r.nbr)
+    # FP32 sums of m terms in sequence carry (m + 1) 2^-24 beside the terms' own error: it counts in the grids of few
+    # cells, where a target has thousands of neighbours
+    most = int(r.nbr.max())
+    check_interaction(g, r, tol=TOL if most < 150 else TOL + (most + 1) * 2.0 ** -24)
 
 
 def test_small_binning_reports_out_of_box_and_recovers():
@@ -66,6 +64,52 @@ def test_small_binning_reports_out_of_box_and_recovers():
         st, mpc = B.pi_sync_status(ctx, s)
         b = oracle.bin_particles(x, y, z, lo, hi, rc)
         assert mpc == b.max_per_cell and np.array_equal(perm.cpu().numpy().view(np.uint32), b.perm)
+    finally:
+        B.pi_destroy(ctx)
+
+
+@pytest.mark.parametrize("n", [1, 1531, 4096])
+@pytest.mark.parametrize("both", [False, True])
+def test_captured_step_with_its_copies(n, both):
+    """Binning, interaction and the copy of the binning results in one graph,
+    replayed on changed positions.  both: two arrays into one destination,
+    which takes memory copies instead of the copying launch."""
+    torch = pytest.importorskip("torch")
+    dev = torch.device("cuda", 0)
+    lo, hi, rc = GRIDS["3375_cells"]
+    ins = [[torch.from_numpy(a).to(dev) for a in W.uniform(n, 60 + k, lo, hi)] for k in range(3)]
+    pos = [t.clone() for t in ins[0]]
+    out = [torch.zeros(n, device=dev) for _ in range(4)] + [torch.zeros(n, dtype=torch.int32, device=dev)
+                                                            for _ in range(2)]
+    ctx = B.pi_create(lo, hi, rc, n)
+
+    def step(s):
+        B.pi_bin(ctx, *pos, n, s)
+        B.pi_interact(ctx, rc / 2, *out[:5], B.PI_ORDER_SORTED, s)
+        B.pi_copy_binned(ctx, perm=out[5], sz=out[5] if both else None, stream=s)
+
+    try:
+        alone = []
+        for t in ins:
+            for p, q in zip(pos, t):
+                p.copy_(q)
+            step(torch.cuda.current_stream())
+            B.pi_sync_status(ctx, torch.cuda.current_stream())
+            alone.append([o.clone() for o in out])
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            step(torch.cuda.current_stream())
+        for k in (1, 2, 0, 2):
+            for o in out:
+                o.zero_()
+            for p, q in zip(pos, ins[k]):
+                p.copy_(q)
+            graph.replay()
+            B.pi_sync_status(ctx, torch.cuda.current_stream())
+            for a, b in zip(out, alone[k]):
+                assert torch.equal(a.view(torch.int32), b.view(torch.int32))
+        b = oracle.bin_particles(*(t.cpu().numpy() for t in ins[2]), lo, hi, rc)
+        assert np.array_equal(out[5].cpu().numpy().view(np.uint32), b.sz.view(np.uint32) if both else b.perm)
     finally:
         B.pi_destroy(ctx)
 
