@@ -20,6 +20,7 @@
 //
 // Every kernel is a dependent launch (see launch_dependent).
 #include <algorithm>
+#include <cstddef>
 #include <mutex>
 
 #include "pi_internal.cuh"
@@ -515,8 +516,6 @@ __global__ void __launch_bounds__(SMALL_THREADS)
 
     for (uint32_t k = tid; k < SMALL_MAX; k += SMALL_THREADS) s_off[k] = 0u;
     pdl_wait();
-    // the control block, cleared before anything can fail a check
-    if (tid < sizeof(Ctrl) / 4) reinterpret_cast<uint32_t*>(ctrl)[tid] = 0u;
     uint32_t c[PER], r[PER];
     bool all_ok = true;
 #pragma unroll
@@ -526,13 +525,12 @@ __global__ void __launch_bounds__(SMALL_THREADS)
         c[j] = i < n ? cell_of(x[i], y[i], z[i], d.g, ok) : 0u;
         all_ok &= ok;
     }
-    // (a barrier too: the counts and the control block are clear)
+    // (a barrier too: the counts are clear)
     const bool ok = __syncthreads_and(all_ok) != 0;
-    bool valid[PER];
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
-        valid[j] = tid + j * SMALL_THREADS < n && PI_BOUNDS(ctrl, c[j], C, CS_HIST_COUNTS);
-        r[j] = valid[j] ? atomicAdd(&s_off[c[j]], 1u) : 0u;
+        const bool valid = tid + j * SMALL_THREADS < n && PI_BOUNDS(ctrl, c[j], C, CS_HIST_COUNTS);
+        r[j] = valid ? atomicAdd(&s_off[c[j]], 1u) : 0u;
     }
     __syncthreads();
     uint32_t v[PER], run = 0, mx = 0;
@@ -574,20 +572,29 @@ __global__ void __launch_bounds__(SMALL_THREADS)
         const uint32_t c0 = tid * PER + 4 * q;
         if (c0 < C) reinterpret_cast<uint4*>(offsets)[c0 / 4] = u;
     }
+    // the control block: every word cleared but the error and M_C
+    constexpr uint32_t ERROR_WORD = offsetof(Ctrl, error) / 4, MAX_WORD = offsetof(Ctrl, max_per_cell) / 4;
+    if (tid < sizeof(Ctrl) / 4)
+        reinterpret_cast<uint32_t*>(ctrl)[tid] =
+            tid == ERROR_WORD ? (ok ? 0u : (uint32_t)ERR_OUT_OF_BOX) : (tid == MAX_WORD ? block_max : 0u);
     if (tid == 0) {
-        if (!ok) atomicOr(&ctrl->error, (uint32_t)ERR_OUT_OF_BOX);
-        ctrl->max_per_cell = block_max;
         pbase[0] = 0u;
         pbase[1] = n;
     }
     for (uint32_t k = tid; k < C; k += SMALL_THREADS) xbins[k] = make_uint2(0u, 0u);
     __syncthreads();
     if (tid == 0) offsets[C] = n;  // (after the padded store of the last group)
+    // the check of the counts once more (debug build): what it found the first
+    // time went with the control block's clearing
+    bool valid[PER];
+#pragma unroll
+    for (int j = 0; j < PER; ++j)
+        valid[j] = tid + j * SMALL_THREADS < n && PI_BOUNDS(ctrl, c[j], C, CS_HIST_COUNTS);
     if (!ok) return;
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
-        if (!valid[j]) continue;
         const uint32_t i = tid + j * SMALL_THREADS;
+        if (!valid[j]) continue;
         const float px = x[i];
         const uint2 t = sub_bin_thermometer(px, c[j], d.g);
         const uint32_t slot = s_off[c[j]] + r[j];
